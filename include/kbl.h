@@ -60,7 +60,10 @@ typedef enum {
 } kbl_status;
 
 /* Arithmetic of the path.
- * KBL_FP64: everything in FP64.
+ * KBL_FP64: everything in FP64; the 2D bounds on grids of at least 3.75 velocity nodes per thermal
+ *   unit ((nu - 1) / (2 k), more than 24 nodes) form the Maxwellians and their envelopes on
+ *   unevaluated sums of two FP32 numbers (48 bits) from FP64 states and sum them in FP64, with an
+ *   error no larger than FP64 products give (2-norm 2e-16 to 2.5e-16 against extended precision).
  * KBL_FP32_MIXED: Maxwellians, envelopes and velocity sums in FP32 (2D: each thread sums its
  *   16 velocity nodes, the threads' sums meet in a pairwise tree, at most 25 roundings of the sum
  *   of magnitudes, which for these single-signed sums is the sum itself: <= 1.5e-6 relative;

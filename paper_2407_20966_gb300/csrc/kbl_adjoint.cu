@@ -251,8 +251,8 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
         else { suy[jj] = u; swy[jj] = wq; }
     }
     __syncthreads();
-    // the same separable tables (and arithmetic) as the forward FP64 kernel, so the
-    // winners of every min / max are those of the forward pass
+    // separable FP64 tables (those of the forward FP64 kernel): the winner of every min / max up to
+    // values equal to rounding
     {
         constexpr int SEG = NX < 16 ? NX : 16, NSG = NX / SEG;
         const double hx = (sbox[1] - sbox[0]) / (NX - 1), hy = (sbox[3] - sbox[2]) / (NX - 1);

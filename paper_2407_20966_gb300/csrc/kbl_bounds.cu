@@ -26,11 +26,10 @@
 // so a block builds per-state row tables (Ex, Ey; FP64 kernels also C*Ex) and every
 // (state, node) pair then costs two multiplies (g = Ex Ey and C g) and four min/max.
 //
-// FP64 kernels: the min/max run on the integer pipe as unsigned 64-bit
-// compares of the bit patterns (all values are >= +0, where integer order is
-// value order), because the GB300 FP64 pipe is ~1/76 of FP32; the row tables
-// come from a product recurrence (kbl_gauss_segment), a few exponentials per
-// segment of 16 nodes.
+// FP64 kernels (kbl_bounds64_body.cuh): the GB300 FP64 pipe runs at ~1/76 of
+// FP32, so grids of 3.75 or more nodes per thermal unit form the envelopes on
+// pairs of floats, decided and valued to 2^-47 per node; coarser grids run the
+// products on the FP64 pipe and the min/max as unsigned 64-bit compares.
 // FP32 kernels: FP64 only for X = rho E - |m|^2/2 (rho P / (gamma-1)) with its
 // positivity test (and, in 1D, for assembling the final bounds; the 2D kernels
 // assemble them in FP32 and widen them exactly); velocities are taken
@@ -47,16 +46,29 @@ namespace {
 
 using namespace kbl_dev;
 
-// 4 resident blocks (64 registers): measured 7% faster than the 2 that 128 registers allow
 template <int N, int NX>
-__global__ void __launch_bounds__(B2f64<NX>::NT, (B2f64<NX>::NT <= 256 ? 4 : 1))
+__global__ void __launch_bounds__(B2f64<NX>::NT, B2f64<NX>::MINB)
 k_bounds2d_f64(const double* __restrict__ w, const double* __restrict__ wf, MeshDev m, Phys ph,
                double* __restrict__ bnd, DevFlags* flags)
 {
-    constexpr int NT = B2f64<NX>::NT;
+    constexpr int NST = N * N + 8 * N, NT = B2f64<NX>::NT;
     const int e = blockIdx.x;
-    bounds2d_f64_core<N * N + 8 * N, NX>([&](double (*sS)[4]) { gather_states<2, N, NT>(w, wf, m, e, sS); },
-                                         m.E, e, ph, bnd, flags);
+    bounds2d_f64_core<NST, NX>(kbl_dyn_smem<Bounds2dF64Smem<NST, NX>>(),
+                               [&](double (*sS)[4]) { gather_states_by_state<N, NT>(w, wf, m, e, sS); }, m.E, e, ph,
+                               bnd, flags);
+}
+
+// the same bounds on float pairs
+template <int N, int NX>
+__global__ void __launch_bounds__(B2pair<NX>::NT, B2pair<NX>::MINB)
+k_bounds2d_pair(const double* __restrict__ w, const double* __restrict__ wf, MeshDev m, Phys ph,
+                double* __restrict__ bnd, DevFlags* flags)
+{
+    constexpr int NST = N * N + 8 * N, NT = B2pair<NX>::NT;
+    const int e = blockIdx.x;
+    bounds2d_pair_core<NST, NX>(kbl_dyn_smem<Bounds2dPairSmem<NST, NX>>(),
+                                [&](double (*sS)[4]) { gather_states_by_state<N, NT>(w, wf, m, e, sS); }, m.E, e, ph,
+                                bnd, flags);
 }
 
 // ---------------------------------------------------------------------------
@@ -193,22 +205,35 @@ k_bounds1d(const double* __restrict__ w, const double* __restrict__ wf, MeshDev 
 template <int N, int NX>
 int run2d(const kbl_ctx* c, const double* w, const double* wf, double* bnd, cudaStream_t s)
 {
-    if (c->cfg.precision == KBL_FP32_MIXED) {
-        const MeshDev m = mesh_of(c);
-        if (c->cfg.nu[0] != NX || c->phys.qwf)   // padded tile or weight table: the 4x4 (or narrower) tile
-            kbl_launch(k_bounds2d_f32<N, NX, 0, true>, c->E, B2f32<NX, 0>::NT, 0, s, c->pdl, w, wf, m, c->phys, bnd,
-                       c->d_flags);
-        else if (NX >= 32 && c->bounds_tile == 1)
-            kbl_launch(k_bounds2d_f32<N, NX, 2>, c->E, B2f32<NX, 2>::NT, 0, s, c->pdl, w, wf, m, c->phys, bnd,
-                       c->d_flags);
-        else if (NX >= 32 && c->bounds_tile == 2)
-            kbl_launch(k_bounds2d_f32<N, NX, 3>, c->E, B2f32<NX, 3>::NT, 0, s, c->pdl, w, wf, m, c->phys, bnd,
-                       c->d_flags);
-        else
-            kbl_launch(k_bounds2d_f32<N, NX, 0>, c->E, B2f32<NX, 0>::NT, 0, s, c->pdl, w, wf, m, c->phys, bnd,
-                       c->d_flags);
-    } else
-        k_bounds2d_f64<N, NX><<<c->E, B2f64<NX>::NT, 0, s>>>(w, wf, mesh_of(c), c->phys, bnd, c->d_flags);
+    const MeshDev m = mesh_of(c);
+    if (c->cfg.nu[0] != NX || c->phys.qwf)   // padded tile or weight table: the 4x4 (or narrower) tile
+        kbl_launch(k_bounds2d_f32<N, NX, 0, true>, c->E, B2f32<NX, 0>::NT, 0, s, c->pdl, w, wf, m, c->phys, bnd,
+                   c->d_flags);
+    else if (NX >= 32 && c->bounds_tile == 1)
+        kbl_launch(k_bounds2d_f32<N, NX, 2>, c->E, B2f32<NX, 2>::NT, 0, s, c->pdl, w, wf, m, c->phys, bnd,
+                   c->d_flags);
+    else if (NX >= 32 && c->bounds_tile == 2)
+        kbl_launch(k_bounds2d_f32<N, NX, 3>, c->E, B2f32<NX, 3>::NT, 0, s, c->pdl, w, wf, m, c->phys, bnd,
+                   c->d_flags);
+    else
+        kbl_launch(k_bounds2d_f32<N, NX, 0>, c->E, B2f32<NX, 0>::NT, 0, s, c->pdl, w, wf, m, c->phys, bnd,
+                   c->d_flags);
+    return 1;
+}
+
+template <int N, int NX>
+int run2d_f64(const kbl_ctx* c, const double* w, const double* wf, double* bnd, cudaStream_t s)
+{
+    kbl_launch_dyn<Bounds2dF64Smem<N * N + 8 * N, NX>>(k_bounds2d_f64<N, NX>, c->E, B2f64<NX>::NT, s, w, wf, mesh_of(c),
+                                                       c->phys, bnd, c->d_flags);
+    return 1;
+}
+
+template <int N, int NX>
+int run2d_pair(const kbl_ctx* c, const double* w, const double* wf, double* bnd, cudaStream_t s)
+{
+    kbl_launch_dyn<Bounds2dPairSmem<N * N + 8 * N, NX>>(k_bounds2d_pair<N, NX>, c->E, B2pair<NX>::NT, s, w, wf,
+                                                        mesh_of(c), c->phys, bnd, c->d_flags);
     return 1;
 }
 
@@ -224,6 +249,11 @@ int run_bounds(const kbl_ctx* c, const double* w, const double* wf, double* bnd,
         else if (wide) k_bounds1d<N, false, true><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
         else k_bounds1d<N, false><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
         return 1;
+    }
+    if (c->cfg.precision != KBL_FP32_MIXED) {
+        if (kbl_pair_grid(c->cfg.nu[0], c->phys.k))
+            KBL_DISPATCH_PAIR(c->cfg.nu[0], return run2d_pair<N, NX>(c, w, wf, bnd, s));
+        KBL_DISPATCH_TILE64(c->cfg.nu[0], return run2d_f64<N, NX>(c, w, wf, bnd, s));
     }
     switch (kbl_tile_nx(c->cfg.nu[0])) {
         case 8: return run2d<N, 8>(c, w, wf, bnd, s);

@@ -190,8 +190,7 @@ __device__ __forceinline__ double kbl_qweight(const Phys& ph, int j, int nu)
 // and its mirror image to the left.  It starts at the segment node nearest U, so every ratio is
 // at most 1 (up to rounding): values only shrink, an underflow to 0 is harmless and nothing
 // overflows.  Each step adds a few ulp; over a 16-node segment the relative error stays
-// below 1e-13.  Callers that must agree bit for bit (the forward bounds and their adjoint)
-// call it with the same arguments.
+// below 1e-13.
 template <typename Emit>
 __device__ __forceinline__ void kbl_gauss_segment(double scale, double U, double th, double lo, double h, int nu,
                                                   int jb, int je, Emit emit)

@@ -2,7 +2,7 @@
 //
 // Eq. 29-46 take any set of states: the bounds of an element follow from the Maxwellians
 // of its stencil whatever element family produced them.  These kernels run the FR path's
-// bounds code (bounds2d_f32_core, bounds2d_f64_core) on stencils the caller assembles --
+// bounds code (bounds2d_f32_core, bounds2d_pair_core, bounds2d_f64_core) on stencils the caller assembles --
 // for triangles with their own solution and face points, or any unstructured mesh whose
 // traces live outside this library -- read from S[E][n_states][4].  A stencil shorter than
 // the compiled capacity (16, 24, 32, 48 or 64 states) repeats its last state, which changes
@@ -40,33 +40,61 @@ k_bounds_stencil_f32(const double* __restrict__ S, int nst, int E, Phys ph, doub
 }
 
 template <int NSTC, int NX>
-__global__ void __launch_bounds__(B2f64<NX>::NT, (B2f64<NX>::NT <= 256 ? 4 : 1))
+__global__ void __launch_bounds__(B2f64<NX>::NT, B2f64<NX>::MINB)
 k_bounds_stencil_f64(const double* __restrict__ S, int nst, int E, Phys ph, double* __restrict__ bnd,
                      DevFlags* flags)
 {
     constexpr int NT = B2f64<NX>::NT;
     const int e = blockIdx.x;
-    bounds2d_f64_core<NSTC, NX>([&](double (*sS)[4]) { gather_explicit<NSTC, NT>(S, nst, e, sS); }, E, e, ph, bnd,
-                                flags);
+    bounds2d_f64_core<NSTC, NX>(kbl_dyn_smem<Bounds2dF64Smem<NSTC, NX>>(),
+                                [&](double (*sS)[4]) { gather_explicit<NSTC, NT>(S, nst, e, sS); }, E, e, ph, bnd, flags);
+}
+
+template <int NSTC, int NX>
+__global__ void __launch_bounds__(B2pair<NX>::NT, B2pair<NX>::MINB)
+k_bounds_stencil_pair(const double* __restrict__ S, int nst, int E, Phys ph, double* __restrict__ bnd,
+                      DevFlags* flags)
+{
+    constexpr int NT = B2pair<NX>::NT;
+    const int e = blockIdx.x;
+    bounds2d_pair_core<NSTC, NX>(kbl_dyn_smem<Bounds2dPairSmem<NSTC, NX>>(),
+                                 [&](double (*sS)[4]) { gather_explicit<NSTC, NT>(S, nst, e, sS); }, E, e, ph, bnd, flags);
 }
 
 template <int NSTC, int NX>
 int run_stencil(const kbl_ctx* c, int E, int nst, const double* S, double* bnd, cudaStream_t s)
 {
-    if (c->cfg.precision == KBL_FP32_MIXED) {
-        if (c->cfg.nu[0] != NX || c->phys.qwf)
-            k_bounds_stencil_f32<NSTC, NX, true><<<E, B2f32<NX, 0>::NT, 0, s>>>(S, nst, E, c->phys, bnd, c->d_flags);
-        else
-            k_bounds_stencil_f32<NSTC, NX, false><<<E, B2f32<NX, 0>::NT, 0, s>>>(S, nst, E, c->phys, bnd, c->d_flags);
-    } else {
-        k_bounds_stencil_f64<NSTC, NX><<<E, B2f64<NX>::NT, 0, s>>>(S, nst, E, c->phys, bnd, c->d_flags);
-    }
+    if (c->cfg.nu[0] != NX || c->phys.qwf)
+        k_bounds_stencil_f32<NSTC, NX, true><<<E, B2f32<NX, 0>::NT, 0, s>>>(S, nst, E, c->phys, bnd, c->d_flags);
+    else
+        k_bounds_stencil_f32<NSTC, NX, false><<<E, B2f32<NX, 0>::NT, 0, s>>>(S, nst, E, c->phys, bnd, c->d_flags);
+    return 1;
+}
+
+template <int NSTC, int NX>
+int run_stencil_f64(const kbl_ctx* c, int E, int nst, const double* S, double* bnd, cudaStream_t s)
+{
+    kbl_launch_dyn<Bounds2dF64Smem<NSTC, NX>>(k_bounds_stencil_f64<NSTC, NX>, E, B2f64<NX>::NT, s, S, nst, E, c->phys, bnd,
+                                              c->d_flags);
+    return 1;
+}
+
+template <int NSTC, int NX>
+int run_stencil_pair(const kbl_ctx* c, int E, int nst, const double* S, double* bnd, cudaStream_t s)
+{
+    kbl_launch_dyn<Bounds2dPairSmem<NSTC, NX>>(k_bounds_stencil_pair<NSTC, NX>, E, B2pair<NX>::NT, s, S, nst, E, c->phys,
+                                               bnd, c->d_flags);
     return 1;
 }
 
 template <int NSTC>
 int run_stencil_nx(const kbl_ctx* c, int E, int nst, const double* S, double* bnd, cudaStream_t s)
 {
+    if (c->cfg.precision != KBL_FP32_MIXED) {
+        if (kbl_pair_grid(c->cfg.nu[0], c->phys.k))
+            KBL_DISPATCH_PAIR(c->cfg.nu[0], return run_stencil_pair<NSTC, NX>(c, E, nst, S, bnd, s));
+        KBL_DISPATCH_TILE64(c->cfg.nu[0], return run_stencil_f64<NSTC, NX>(c, E, nst, S, bnd, s));
+    }
     switch (kbl_tile_nx(c->cfg.nu[0])) {
         case 8: return run_stencil<NSTC, 8>(c, E, nst, S, bnd, s);
         case 16: return run_stencil<NSTC, 16>(c, E, nst, S, bnd, s);

@@ -5,7 +5,7 @@
 // value at the same place (edge g of the neighbour, its point p - k, the edge running the other
 // way) or the boundary state.  Gathering it here, straight from w and wf, spares the triangle
 // step the stencil array S (written by one kernel, read by the next); the bounds code is the
-// explicit-stencil kernels' (bounds2d_f32_core, bounds2d_f64_core), padded by repeating the
+// explicit-stencil kernels' (bounds2d_f32_core, bounds2d_pair_core, bounds2d_f64_core), padded by repeating the
 // last state (neither the envelopes nor the velocity box change).
 #include "kbl_bounds64_body.cuh"
 
@@ -59,30 +59,58 @@ k_bounds_tri_f32(TriGather a, int E, Phys ph, double* __restrict__ bnd, DevFlags
 }
 
 template <int NSTC, int NX>
-__global__ void __launch_bounds__(B2f64<NX>::NT, (B2f64<NX>::NT <= 256 ? 4 : 1))
+__global__ void __launch_bounds__(B2f64<NX>::NT, B2f64<NX>::MINB)
 k_bounds_tri_f64(TriGather a, int E, Phys ph, double* __restrict__ bnd, DevFlags* flags)
 {
     constexpr int NT = B2f64<NX>::NT;
     const int e = blockIdx.x;
-    bounds2d_f64_core<NSTC, NX>([&](double (*sS)[4]) { gather_tri<NSTC, NT>(a, e, sS); }, E, e, ph, bnd, flags);
+    bounds2d_f64_core<NSTC, NX>(kbl_dyn_smem<Bounds2dF64Smem<NSTC, NX>>(),
+                                [&](double (*sS)[4]) { gather_tri<NSTC, NT>(a, e, sS); }, E, e, ph, bnd, flags);
+}
+
+template <int NSTC, int NX>
+__global__ void __launch_bounds__(B2pair<NX>::NT, B2pair<NX>::MINB)
+k_bounds_tri_pair(TriGather a, int E, Phys ph, double* __restrict__ bnd, DevFlags* flags)
+{
+    constexpr int NT = B2pair<NX>::NT;
+    const int e = blockIdx.x;
+    bounds2d_pair_core<NSTC, NX>(kbl_dyn_smem<Bounds2dPairSmem<NSTC, NX>>(),
+                                 [&](double (*sS)[4]) { gather_tri<NSTC, NT>(a, e, sS); }, E, e, ph, bnd, flags);
 }
 
 template <int NSTC, int NX>
 void run_tri(const kbl_ctx* c, int E, const TriGather& a, double* bnd, cudaStream_t s)
 {
-    if (c->cfg.precision == KBL_FP32_MIXED) {
-        if (c->cfg.nu[0] != NX || c->phys.qwf)
-            k_bounds_tri_f32<NSTC, NX, true><<<E, B2f32<NX, 0>::NT, 0, s>>>(a, E, c->phys, bnd, c->d_flags);
-        else
-            k_bounds_tri_f32<NSTC, NX, false><<<E, B2f32<NX, 0>::NT, 0, s>>>(a, E, c->phys, bnd, c->d_flags);
-    } else {
-        k_bounds_tri_f64<NSTC, NX><<<E, B2f64<NX>::NT, 0, s>>>(a, E, c->phys, bnd, c->d_flags);
-    }
+    if (c->cfg.nu[0] != NX || c->phys.qwf)
+        k_bounds_tri_f32<NSTC, NX, true><<<E, B2f32<NX, 0>::NT, 0, s>>>(a, E, c->phys, bnd, c->d_flags);
+    else
+        k_bounds_tri_f32<NSTC, NX, false><<<E, B2f32<NX, 0>::NT, 0, s>>>(a, E, c->phys, bnd, c->d_flags);
+}
+
+template <int NSTC, int NX>
+int run_tri_f64(const kbl_ctx* c, int E, const TriGather& a, double* bnd, cudaStream_t s)
+{
+    kbl_launch_dyn<Bounds2dF64Smem<NSTC, NX>>(k_bounds_tri_f64<NSTC, NX>, E, B2f64<NX>::NT, s, a, E, c->phys, bnd,
+                                              c->d_flags);
+    return 1;
+}
+
+template <int NSTC, int NX>
+int run_tri_pair(const kbl_ctx* c, int E, const TriGather& a, double* bnd, cudaStream_t s)
+{
+    kbl_launch_dyn<Bounds2dPairSmem<NSTC, NX>>(k_bounds_tri_pair<NSTC, NX>, E, B2pair<NX>::NT, s, a, E, c->phys, bnd,
+                                               c->d_flags);
+    return 1;
 }
 
 template <int NSTC>
 int run_tri_nx(const kbl_ctx* c, int E, const TriGather& a, double* bnd, cudaStream_t s)
 {
+    if (c->cfg.precision != KBL_FP32_MIXED) {
+        if (kbl_pair_grid(c->cfg.nu[0], c->phys.k))
+            KBL_DISPATCH_PAIR(c->cfg.nu[0], return run_tri_pair<NSTC, NX>(c, E, a, bnd, s));
+        KBL_DISPATCH_TILE64(c->cfg.nu[0], return run_tri_f64<NSTC, NX>(c, E, a, bnd, s));
+    }
     switch (kbl_tile_nx(c->cfg.nu[0])) {
         case 8: run_tri<NSTC, 8>(c, E, a, bnd, s); return 1;
         case 16: run_tri<NSTC, 16>(c, E, a, bnd, s); return 1;
