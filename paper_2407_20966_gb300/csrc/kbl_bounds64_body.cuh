@@ -305,9 +305,9 @@ __device__ __forceinline__ void bounds2d_f64_core(Bounds2dF64Smem<NST, NX>& sm, 
 // are formed on unevaluated sums of two floats (hi + lo, 48-49 significant bits) and the FP64 pipe
 // keeps what decides the result's accuracy per state (the primitive state, the velocity box, the
 // exponents' coefficients) and per sum (the moments).  Errors against extended precision (2-norm; the
-// kernel above in brackets, its tables drift along the recurrence): vortex 2.4e-16 (2.8e-16), smooth
-// waves 2.3e-16 (2.6e-16), blast 2.5e-16 (4.4e-16), scattered states 2.2e-16 (2.3e-16), 64 nodes
-// 2.4e-16 (4.4e-16).
+// kernel above in brackets, its tables drift along the recurrence): vortex 2.1e-16 (2.8e-16), smooth
+// waves 2.0e-16 (2.6e-16), blast 2.2e-16 (4.4e-16), scattered states 2.1e-16 (2.3e-16), 64 nodes
+// 1.7e-16 (4.4e-16), 33 nodes by Romberg 2.7e-16 (2.6e-16).
 //
 //   row tables   a_i(u) = A_i 2^-t(u), c_i = C_i a_i, b_i(v) = 2^-t(v), t = (u - U)^2 log2(e)/(2 theta),
 //                t in 64-bit fixed point by second differences (exact additions), 2^-t by a table of
@@ -316,10 +316,13 @@ __device__ __forceinline__ void bounds2d_f64_core(Bounds2dF64Smem<NST, NX>& sm, 
 //   pass 2       E = max_i [a_hi b_hi - M + a_hi b_lo + a_lo b_hi] by FMAs, the first of which forms
 //                a_hi b_hi - M with one rounding: the envelope is M + E, its winner decided to
 //                2^-47, its value off by as little
-//   moments      in FP64; the quadrature weights are in the tables already
+//   moments      the nodes' values in error-free FP32 sums along rows and columns, those in FP64;
+//                the quadrature weights are in the tables already
 //
-// Measured at 128^2 P3, 32^2 grid: 1.08 ms per launch, 6.52 ms for the FP64 kernel above (86% of the
-// FP64 pipe); 33^2 Romberg grid (46 x 27 P4): 0.25 ms on a 40-node tile, 2.77 ms on the FP64 kernel's 64.
+// Measured at 128^2 P3, 32^2 grid: 0.95 ms per launch (1.08 ms with the moments node by node in FP64 and
+// the states' constants in two passes over shared memory), 6.52 ms for the FP64 kernel above (86% of
+// the FP64 pipe); 33^2 Romberg grid (46 x 27 P4): 0.24 ms on a 40-node tile, 2.77 ms on the FP64
+// kernel's 64.
 // What bounds it: per (state, node) 14 FP32 products/FMAs (packed two to an instruction, two
 // neighbouring x nodes) and four three-input min/max, 7 + 4 issue slots.
 //
@@ -443,7 +446,7 @@ __device__ __forceinline__ void exp2_reduce(long long t, const float2* kT, const
 
 // y = 2^-(t + n) for t in units of 2^-55, 0 <= t < 256: n the whole part (rounded to 1/128); two at a
 // time.  2^-r - 1 of the remainder |r| <= 2^-8 by its Taylor series on float pairs.  Against extended
-// precision h + l is 0.73 2^-50 off (rms; a correctly rounded pair 0.64 2^-50), max 3.2 2^-50.
+// precision h + l is 0.65 2^-50 off (rms; a correctly rounded pair 0.64 2^-50), max 2.5 2^-50.
 __device__ __forceinline__ Triple2 exp2_pair(long long t0, long long t1, const float2* kT, const int* kF, int& n0, int& n1)
 {
     float2 T0, T1, rh, rl;
@@ -463,6 +466,7 @@ __device__ __forceinline__ Triple2 exp2_pair(long long t0, long long t1, const f
     float2 qe = __ffma2_rn(C2H, s, f2neg(q));
     qe = __ffma2_rn(C2L, s, qe);
     qe = __ffma2_rn(C2H, se, qe);
+    qe = __ffma2_rn(f2dup(-0.16651233f), __fmul2_rn(s, rl), qe);   // the cube's -ln^3 2 / 2 r_hi^2 r_lo
     // -ln^3 2 / 6 + ln^4 2 / 24 r - ln^5 2 / 120 r^2
     const float2 g = __ffma2_rn(__ffma2_rn(f2dup(-0.0013333558f), rh, f2dup(0.009618129f)), rh, f2dup(-0.05550411f));
     const float2 cub = __fmul2_rn(__fmul2_rn(s, rh), g);
@@ -486,17 +490,35 @@ __device__ __forceinline__ void triple_store(const Triple2& y, float2 sc, float2
     carry = f2sub(rt, f2sub(l, lt));
 }
 
-// x in units of 2^-58, rounded; |x| < 16.
+// x in units of 2^-58, rounded; |x| < 32.
 __device__ __forceinline__ long long fixed58(double x)
 {
     const long long b = __double_as_longlong(x);
     const int ex = (int)((b >> 52) & 0x7ff) - 1017;     // the significand's shift
     const long long m = (b & 0xfffffffffffffll) | (1ll << 52);
     long long v;
-    if (ex >= 0) v = m << min(ex, 9);
+    if (ex >= 0) v = m << min(ex, 10);
     else if (ex > -54) v = (m + (1ll << (-ex - 1))) >> -ex;
     else v = 0;
     return b < 0 ? -v : v;
+}
+
+// Whether x > 0 lies within 2^+-900.
+__device__ __forceinline__ bool exponent_ok(double x) { return (unsigned)((__double2hiint(x) >> 20) - 123) <= 1800u; }
+
+// a / b from inv = 1 / b correctly rounded: the corrected product is the correctly rounded quotient
+// (Markstein) while nothing over- or underflows.
+__device__ __forceinline__ double quotient_of(double a, double b, double inv)
+{
+    const double t = a * inv;
+    return fma(fma(-t, b, a), inv, t);
+}
+
+// What rs = rsqrt(x), rounded, misses of 1 / sqrt(x).
+__device__ __forceinline__ double rsqrt_rest(double x, double rs)
+{
+    const double r2 = rs * rs;
+    return (0.5 * rs) * fma(-x, fma(rs, rs, -r2), fma(-x, r2, 1.0));
 }
 
 // x as the nearest float, the rest's, and the rest's.
@@ -504,9 +526,9 @@ __device__ __forceinline__ Triple split_f32(double x)
 {
     Triple t;
     t.h = (float)x;
-    const double e = x - (double)t.h;
+    const double e = x - f64_widen(t.h);
     t.l = (float)e;
-    t.r = (float)(e - (double)t.l);
+    t.r = (float)(e - f64_widen(t.l));
     return t;
 }
 
@@ -550,7 +572,7 @@ struct Bounds2dPairSmem {
         } tab;
         F64Tables<NST, NX, NW> gen;   // an element out of the pairs' range
     } u;
-    double S[NST][4];                 // the stencil; then rho / theta, theta, U
+    double S[NST][4];                 // the stencil
     PairState P[NST];
     float2 kT[128];                   // kbl_exp2_knots
     int kF[128];
@@ -560,7 +582,7 @@ struct Bounds2dPairSmem {
     Triple q[NX];                     // quadrature weights (a table's: the trapezoidal ones are in the code)
     long long kbox[NW][4];
     int kmax[NW];
-    double lo[2], hi[2], h[2];        // velocity box and grid spacing per axis
+    double lo[2], hi[2], h[2], c[2];  // velocity box, grid spacing and node (nu - 1) / 2 per axis
 };
 
 template <int NST, int NX>
@@ -578,6 +600,63 @@ __device__ __forceinline__ double widen_fast(float x)
     return __hiloint2double(((b >> 3) & (int)0x8fffffff) + 0x38000000, b << 29);
 }
 
+// Column k of the warps' sums, pairwise: one after the other their roundings add up at full size.
+template <int NW>
+__device__ __forceinline__ double sum_warps(const double (*red)[8], int k)
+{
+    double a[NW];
+#pragma unroll
+    for (int q = 0; q < NW; q++) a[q] = red[q][k];
+#pragma unroll
+    for (int d = 1; d < NW; d *= 2)
+#pragma unroll
+        for (int q = 0; q + d < NW; q += 2 * d) a[q] += a[q + d];
+    return a[0];
+}
+
+// Sums of envelope values -M + E (the passes keep the negated M): -m - e + r + q with m the FP32 sum of
+// the M, e its error, r the FP32 sum of the E, q its error.
+struct Sum4 {
+    float m, e, r, q;
+    __device__ __forceinline__ double value() const
+    {
+        return (widen_fast(-m) + widen_fast(-e)) + (widen_fast(r) + widen_fast(q));
+    }
+};
+struct Sum4x2 {
+    float2 m, e, r, q;
+};
+// without q (two summands: one rounding)
+struct Sum3 {
+    float m, e, r;
+    __device__ __forceinline__ double value() const { return (widen_fast(-m) + widen_fast(-e)) + widen_fast(r); }
+};
+__device__ __forceinline__ Sum4x2 sum_pairs(float2 Ma, float2 Ea, float2 Mb, float2 Eb)
+{
+    Sum4x2 s;
+    f2two_sum(Ma, Mb, s.m, s.e);
+    f2two_sum(Ea, Eb, s.r, s.q);
+    return s;
+}
+__device__ __forceinline__ Sum4x2 sum_sums(const Sum4x2& a, const Sum4x2& b)
+{
+    Sum4x2 s;
+    f2two_sum(a.m, b.m, s.m, s.e);
+    s.e = __fadd2_rn(s.e, __fadd2_rn(a.e, b.e));
+    f2two_sum(a.r, b.r, s.r, s.q);
+    s.q = __fadd2_rn(s.q, __fadd2_rn(a.q, b.q));
+    return s;
+}
+__device__ __forceinline__ Sum4 sum_lanes(const Sum4x2& a)
+{
+    Sum4 s;
+    two_sum(a.m.x, a.m.y, s.m, s.e);
+    s.e = __fadd_rn(s.e, __fadd_rn(a.e.x, a.e.y));
+    two_sum(a.r.x, a.r.y, s.r, s.q);
+    s.q = __fadd_rn(s.q, __fadd_rn(a.q.x, a.q.y));
+    return s;
+}
+
 // 2^k for |k| <= 1000
 __device__ __forceinline__ double pow2_f64(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
@@ -592,49 +671,50 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
     constexpr int NT = SH::NT, NW = SM::NW, NSTP = SM::NSTP, TX = SH::TX, TY = SH::TY;
     static_assert(TX == 4, "two packed pairs of x nodes per thread");
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    static_assert(NST <= NT, "a thread per state");
     const int nu = ph.nu[0];   // nodes per axis; tile nodes j >= nu carry no weight
-    gather(sm.S);
+    gather(sm.S);              // thread i fills S[i]
     for (int k = tid; k < 128; k += NT) {
         const Exp2Knot q = kbl_exp2_knots[k];
         sm.kT[k] = make_float2(__uint_as_float(q.hi), __uint_as_float(q.lo));
         sm.kF[k] = q.f;
     }
-    __syncthreads();
 
-    // 1. primitive states in FP64; one reciprocal per quotient's divisor and a corrected quotient
+    // 1. primitive states in FP64, one thread each.  With inv = 1 / rho correctly rounded, the
+    //    corrected product a inv is the correctly rounded a / rho (Markstein), within the exponent
+    //    range checked first.
     long long klo[2] = {0x7fffffffffffffffll, 0x7fffffffffffffffll}, khi[2] = {-0x7fffffffffffffffll, -0x7fffffffffffffffll};
-    int kA = 0;
-    int bad = 0;
-    for (int i = tid; i < NST; i += NT) {
-        const double* q = sm.S[i];
-        const double rho = q[0], P = kbl_pressure<2>(q, ph.gamma - 1.0);
-        if (!(rho > 0.0) || !(P > 0.0)) bad = 1;
-        const double inv = 1.0 / rho;
-        double th = P * inv, ux = q[1] * inv, uy = q[2] * inv;
-        th = fma(fma(-th, rho, P), inv, th);
-        ux = fma(fma(-ux, rho, q[1]), inv, ux);
-        uy = fma(fma(-uy, rho, q[2]), inv, uy);
-        const double rs = rsqrt(th);
-        double sq = th * rs;
-        sq = fma(fma(-sq, sq, th), 0.5 * rs, sq);
-        const double ksq = ph.k * sq;
-        double A = rho * (rs * rs);                 // rho / theta (1 / (2 pi) is in the exponents)
-        A = fma(fma(-A, th, rho), rs * rs, A);
-        sm.S[i][0] = A;
-        sm.S[i][1] = th;
-        sm.S[i][2] = ux;
-        sm.S[i][3] = uy;
-        klo[0] = min(klo[0], key64(ux - ksq)); khi[0] = max(khi[0], key64(ux + ksq));
-        klo[1] = min(klo[1], key64(uy - ksq)); khi[1] = max(khi[1], key64(uy + ksq));
-        kA = max(kA, __double2hiint(A));
-    }
-    // a bad state leaves the block at once, as a whole
-    if (__syncthreads_or(bad)) {
-        if (tid == 0) {
-            write_nan(bnd, E, e, 4);
-            atomicOr(&flags->nonphysical, 1);
+    int kA = 0, bad = 0, out_of_range = 0;
+    double th = 0.0, rs = 0.0, U[2] = {0.0, 0.0}, A = 0.0;
+    if (tid < NST) {
+        const double rho = sm.S[tid][0], mx = sm.S[tid][1], my = sm.S[tid][2], En = sm.S[tid][3];
+        if (exponent_ok(rho) && exponent_ok(En)) {
+            const double inv = 1.0 / rho;
+            auto over_rho = [&](double a) { return quotient_of(a, rho, inv); };
+            double mm = mx * mx;
+            mm += my * my;
+            const double P = (ph.gamma - 1.0) * (En - over_rho(0.5 * mm));
+            bad = !(P > 0.0);
+            th = over_rho(P);
+            U[0] = over_rho(mx);
+            U[1] = over_rho(my);
+            rs = rsqrt(th);
+            double sq = th * rs;
+            sq = fma(fma(-sq, sq, th), 0.5 * rs, sq);
+            const double it = rs * rs;
+            A = rho * it;                           // rho / theta (1 / (2 pi) is in the exponents)
+            A = fma(fma(-A, th, rho), it, A);
+#pragma unroll
+            for (int d = 0; d < 2; d++) {
+                klo[d] = key64(fma(-ph.k, sq, U[d]));
+                khi[d] = key64(fma(ph.k, sq, U[d]));
+            }
+            kA = __double2hiint(A);
+            out_of_range = !exponent_ok(th);
+        } else {
+            bad = !(rho > 0.0) || !(kbl_pressure<2>(sm.S[tid], ph.gamma - 1.0) > 0.0);
+            out_of_range = 1;
         }
-        return;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -650,7 +730,13 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
         sm.kbox[wid][2] = klo[1]; sm.kbox[wid][3] = khi[1];
         sm.kmax[wid] = kA;
     }
-    __syncthreads();
+    if (__syncthreads_or(bad)) {
+        if (tid == 0) {
+            write_nan(bnd, E, e, 4);
+            atomicOr(&flags->nonphysical, 1);
+        }
+        return;
+    }
     if (tid < 2) {
         long long a = sm.kbox[0][2 * tid], b = sm.kbox[0][2 * tid + 1];
 #pragma unroll
@@ -659,9 +745,11 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
             b = max(b, sm.kbox[q][2 * tid + 1]);
         }
         const double la = unkey64(a), lb = unkey64(b);
+        const double hd = (lb - la) / (nu - 1);
         sm.lo[tid] = la;
         sm.hi[tid] = lb;
-        sm.h[tid] = (lb - la) / (nu - 1);
+        sm.h[tid] = hd;
+        sm.c[tid] = fma((double)((nu - 1) / 2), hd, la);
     }
     kA = sm.kmax[0];
 #pragma unroll
@@ -674,49 +762,43 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
     for (int d = 0; d < 2; d++)
         kU = max(kU, max(__double2hiint(sm.lo[d]) & 0x7fffffff, __double2hiint(sm.hi[d]) & 0x7fffffff));
     const int eU = (kU >> 20) - 1022;
-    int out_of_range = (abs(eA) > 900) | (abs(eU) > 450);
-    const double sA = pow2_f64(out_of_range ? 0 : -eA), sU = pow2_f64(out_of_range ? 0 : -eU);
+    if (abs(eA) > 900 || abs(eU) > 450) out_of_range = 1;
+    const double sA = pow2_f64(abs(eA) > 900 ? 0 : -eA), sU = pow2_f64(abs(eU) > 450 ? 0 : -eU);
 
     // 2. scaled constants, and the velocity grid's coefficients
-    for (int i = tid; i < NST; i += NT) {
-        const double th = sm.S[i][1], rs = rsqrt(th);
-        const Triple A = split_f32(sm.S[i][0] * sA);
-        const Triple C = split_f32(0.5 * (2.0 / (ph.gamma - 1.0) - 2) * th * (sU * sU));
+    if (tid < NST) {
+        const Triple At = split_f32(A * sA), Ct = split_f32(ph.half_delta2 * th * (sU * sU));
         // kappa = sqrt(log2(e) / 2) / sqrt(theta) as kh + kl
-        const double r2 = rs * rs;
-        const double rl = 0.5 * rs * (fma(-th, r2, 1.0) - th * fma(rs, rs, -r2));
+        const double rl = rsqrt_rest(th, rs);
         const double kh = 0.8493218002880191 * rs;
         const double kl = fma(0.8493218002880191, rs, -kh) + fma(-2.5959464104597403e-17, rs, 0.8493218002880191 * rl);
         float tm = 0.0f;
 #pragma unroll
         for (int d = 0; d < 2; d++) {
-            const double hd = sm.h[d], dc = fma((double)((nu - 1) / 2), hd, sm.lo[d]) - sm.S[i][2 + d];
+            const double hd = sm.h[d], dc = sm.c[d] - U[d];
             const double zh = dc * kh, dh = hd * kh;
             // the low parts, below 2^-48, in units of 2^-58 like the high ones
-            const double zl = fma(dc, kh, -zh) + dc * kl, dl = fma(hd, kh, -dh) + hd * kl;
-            sm.P[i].z[d] = fixed58(zh) + fixed58(zl);
-            sm.P[i].dz[d] = fixed58(dh) + fixed58(dl);
+            const double zl = fma(dc, kl, fma(dc, kh, -zh)), dl = fma(hd, kl, fma(hd, kh, -dh));
+            sm.P[tid].z[d] = fixed58(zh) + fixed58(zl);
+            sm.P[tid].dz[d] = fixed58(dh) + fixed58(dl);
             // the largest exponent over the box, in FP32 with a margin
-            const float z = f32_trunc(zh), dz = f32_trunc(dh) * (float)(nu / 2 + 1);
-            tm = fmaxf(tm, fabsf(z) + dz);
+            tm = fmaxf(tm, fabsf(f32_trunc(zh)) + f32_trunc(dh) * (float)(nu / 2 + 1));
         }
-        sm.P[i].A = A;
-        sm.P[i].C = C;
-        if (!(tm < 15.5f) || !(A.h >= 0x1p-60f) || !(C.h == 0.0f || (C.h >= 0x1p-30f && C.h < 0x1p60f))) out_of_range = 1;
+        sm.P[tid].A = At;
+        sm.P[tid].C = Ct;
+        if (!(tm < 15.5f) || !(At.h >= 0x1p-60f) || !(Ct.h == 0.0f || (Ct.h >= 0x1p-30f && Ct.h < 0x1p60f))) out_of_range = 1;
     }
-    for (int j = tid; j < 2 * NX; j += NT) {
+    for (int j = NT - 1 - tid; j < 2 * NX; j += NT) {   // from the last thread: the first hold states
         const int d = j / NX, jj = j % NX;
         const double u = sm.lo[d] + min(jj, nu - 1) * sm.h[d];
         const double us = u * sU;
-        const bool neg = us < 0.0;
+        const bool neg = __double2hiint(us) < 0;
         sm.wt[d][0][jj] = us * (neg ? ph.rel_hi : ph.rel_lo);
         sm.wt[d][1][jj] = us * (neg ? ph.rel_lo : ph.rel_hi);
         sm.wt[d][2][jj] = 0.5 * us * us;
         if (ph.qw && d == 0) sm.q[jj] = split_f32(kbl_qweight(ph, jj, nu));
     }
     if (__syncthreads_or(out_of_range)) {
-        gather(sm.S);
-        __syncthreads();
         bounds2d_pair_redo<NST, NX>(sm, E, e, ph, bnd, flags);
         return;
     }
@@ -724,7 +806,7 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
     // 3. row tables: runs of 8 nodes, t by second differences
     constexpr int SEG = 8, NSG = NX / SEG;
     for (int task = tid; task < NSTP * 2 * NSG; task += NT) {
-        const int i = task / (2 * NSG), axis = (task / NSG) & 1, jb = (task % NSG) * SEG;
+        const int axis = task >= NSTP * NSG, i = (task / NSG) % NSTP, jb = (task % NSG) * SEG;   // x rows first
         const PairState& s = sm.P[i < NST ? i : NST - 1];
         // t = z^2 and its differences in units of 2^-55, rounded to nearest (their errors add up over
         // the run; the tail of a padded tile may wrap: it carries no weight)
@@ -865,37 +947,59 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
             }
         }
 
-        // 5. moments of the thread's nodes in FP64
+        // 5. moments: the envelopes' two floats meet in error-free FP32 sums (a row over x for the weights
+        //    in v, a column over y for those in u, everything for I), which then enter FP64: a third of
+        //    the FP64 instructions that node by node takes (8.4k clocks per element on that pipe before)
+        Sum4 V[TY][2], I[2];
+        Sum3 C[TX][2];
 #pragma unroll
-        for (int a = 0; a < TX; a++) {
-            const int p = a >> 1;
-            auto lane_of = [&](float2 v) { return (a & 1) ? v.y : v.x; };
-            double cT[2] = {0.0, 0.0};
+        for (int s = 0; s < 2; s++) {
 #pragma unroll
             for (int b = 0; b < TY; b++) {
-                const int jy = ty * TY + b;
-                const double T0 = widen_fast(lane_of(etl[b][p])) - widen_fast(lane_of(tlo[b][p]));
-                const double T1 = widen_fast(lane_of(eth[b][p])) - widen_fast(lane_of(thi[b][p]));
-                const double I0 = widen_fast(lane_of(eil[b][p])) - widen_fast(lane_of(ilo[b][p]));
-                const double I1 = widen_fast(lane_of(eih[b][p])) - widen_fast(lane_of(ihi[b][p]));
-                const double v0 = sm.wt[1][0][jy], v1 = sm.wt[1][1][jy], kv = sm.wt[1][2][jy];
-                const bool neg = __double2hiint(v0) < 0;   // v < 0: the lower sum takes the upper envelope
-                cT[0] = b == 0 ? T0 : cT[0] + T0;
-                cT[1] = b == 0 ? T1 : cT[1] + T1;
-                acc[4] = fma(v0, neg ? T1 : T0, acc[4]);
-                acc[5] = fma(v1, neg ? T0 : T1, acc[5]);
-                acc[6] = fma(kv, T0, acc[6]) + I0;
-                acc[7] = fma(kv, T1, acc[7]) + I1;
+                const float2(&M)[2] = s ? thi[b] : tlo[b];
+                const float2(&r)[2] = s ? eth[b] : etl[b];
+                V[b][s] = sum_lanes(sum_pairs(M[0], r[0], M[1], r[1]));
             }
+            Sum4x2 ci[2];
+#pragma unroll
+            for (int p = 0; p < 2; p++) {
+                float2 m, e;
+                f2two_sum(s ? thi[0][p] : tlo[0][p], s ? thi[1][p] : tlo[1][p], m, e);
+                const float2 r = __fadd2_rn(s ? eth[0][p] : etl[0][p], s ? eth[1][p] : etl[1][p]);
+                C[2 * p][s] = Sum3{m.x, e.x, r.x};
+                C[2 * p + 1][s] = Sum3{m.y, e.y, r.y};
+                ci[p] = s ? sum_pairs(ihi[0][p], eih[0][p], ihi[1][p], eih[1][p])
+                          : sum_pairs(ilo[0][p], eil[0][p], ilo[1][p], eil[1][p]);
+            }
+            I[s] = sum_lanes(sum_sums(ci[0], ci[1]));
+        }
+        double vs[TY][2];
+#pragma unroll
+        for (int b = 0; b < TY; b++) {
+            const int jy = ty * TY + b;
+            const double v0 = sm.wt[1][0][jy], v1 = sm.wt[1][1][jy], kv = sm.wt[1][2][jy];
+            const bool neg = __double2hiint(v0) < 0;   // v < 0: the lower sum takes the upper envelope
+#pragma unroll
+            for (int s = 0; s < 2; s++) vs[b][s] = V[b][s].value();
+            acc[4] = fma(v0, neg ? vs[b][1] : vs[b][0], acc[4]);
+            acc[5] = fma(v1, neg ? vs[b][0] : vs[b][1], acc[5]);
+            acc[6] = fma(kv, vs[b][0], acc[6]);
+            acc[7] = fma(kv, vs[b][1], acc[7]);
+        }
+        acc[0] = vs[0][0] + vs[1][0];
+        acc[1] = vs[0][1] + vs[1][1];
+        acc[6] += I[0].value();
+        acc[7] += I[1].value();
+#pragma unroll
+        for (int a = 0; a < TX; a++) {
             const int jx = 4 * tx + a;
             const double u0 = sm.wt[0][0][jx], u1 = sm.wt[0][1][jx], ku = sm.wt[0][2][jx];
             const bool neg = __double2hiint(u0) < 0;
-            acc[0] += cT[0];
-            acc[1] += cT[1];
-            acc[2] = fma(u0, neg ? cT[1] : cT[0], acc[2]);
-            acc[3] = fma(u1, neg ? cT[0] : cT[1], acc[3]);
-            acc[6] = fma(ku, cT[0], acc[6]);
-            acc[7] = fma(ku, cT[1], acc[7]);
+            const double c0 = C[a][0].value(), c1 = C[a][1].value();
+            acc[2] = fma(u0, neg ? c1 : c0, acc[2]);
+            acc[3] = fma(u1, neg ? c0 : c1, acc[3]);
+            acc[6] = fma(ku, c0, acc[6]);
+            acc[7] = fma(ku, c1, acc[7]);
         }
     }
     // 6. warp reduce-scatter of the eight sums (lane 4 k holds sum k), then the warps
@@ -916,20 +1020,19 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
     __syncthreads();
     int redo = 0;
     if (tid < 8) {
-        double s = 0.0;
-#pragma unroll
-        for (int q = 0; q < NW; q++) s += sm.red[q][tid];
+        double s = sum_warps<NW>(sm.red, tid);
         // sum k: rho, m_x, m_y, E (k >> 1), lower then upper
         const int v = tid >> 1, up = tid & 1;
         if (tid == 0 && !(s >= 0x1p-40)) redo = 1;
-        double val = s * (sm.h[0] * sm.h[1] * pow2_f64(eA)) * (v == 0 ? 1.0 : v == 3 ? pow2_f64(2 * eU) : pow2_f64(eU));
-        if (v == 0 || v == 3) val *= up ? ph.rel_hi : ph.rel_lo;
+        // times h_x h_y and the relaxation (in the momentum weights already), rounded once
+        const double hh = sm.h[0] * sm.h[1], p = s * hh;
+        const double rest = fma(s, fma(sm.h[0], sm.h[1], -hh), fma(s, hh, -p));
+        const double rel = v == 0 || v == 3 ? (up ? ph.rel_hi : ph.rel_lo) : 1.0;
+        double val = fma(rel, p, rel * rest) * pow2_f64(eA) * (v == 0 ? 1.0 : v == 3 ? pow2_f64(2 * eU) : pow2_f64(eU));
         if (tid == 0 && val < ph.rho_floor) val = ph.rho_floor;
         bnd[((size_t)up * 4 + v) * E + e] = val;
     }
     if (__syncthreads_or(redo)) {
-        gather(sm.S);
-        __syncthreads();
         bounds2d_pair_redo<NST, NX>(sm, E, e, ph, bnd, flags);
     }
 }

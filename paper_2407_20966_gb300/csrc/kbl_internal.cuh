@@ -64,7 +64,7 @@ struct Phys {
     // derived on the host (kbl_phys_derive), so that FP32 kernels spend no FP64 division or
     // conversion on them: gamma - 1, k, delta / 2 = 1/(gamma - 1) - d/2 for d = 2, 1 -+ r
     float gm1f, kf, half_delta2f;
-    double rel_lo, rel_hi;
+    double rel_lo, rel_hi, half_delta1, half_delta2;   // delta / 2 for d = 1, 2
     float rel_lof, rel_hif;   // FP32 copies of 1 -+ r
     // float bounds for the limiter's FP32 screen: eps and p_floor rounded up, gamma - 1 down
     float epsf_up, pfloorf_up, gm1f_down;
@@ -75,6 +75,8 @@ inline void kbl_phys_derive(Phys& p)
     p.gm1f = (float)(p.gamma - 1.0);
     p.kf = (float)p.k;
     p.half_delta2f = 0.5f * (float)(2.0 / (p.gamma - 1.0) - 2.0);
+    p.half_delta1 = 0.5 * (2.0 / (p.gamma - 1.0) - 1);
+    p.half_delta2 = 0.5 * (2.0 / (p.gamma - 1.0) - 2);
     p.epsf_up = kbl_f32_up(p.eps);
     p.pfloorf_up = kbl_f32_up(p.p_floor);
     p.gm1f_down = kbl_f32_down(p.gamma - 1.0);
