@@ -85,15 +85,43 @@ k_bounds2d_f32(const double* __restrict__ w, const double* __restrict__ wf, Mesh
 }
 
 // ---------------------------------------------------------------------------
-// 1D (FP64 and FP32): one block per element, one thread per velocity node
-// (strided), direct evaluation of every Maxwellian.
+// 1D, FP64: one block per element, the velocity nodes over its threads (kbl_bounds64_body.cuh).  Bound by
+// instruction issue; an FP64 exponential and quotient per (state, node) held the FP64 pipe 42 slots
+// each: 374 -> 75 us per launch at 300 P4 elements, 2048 nodes, 23 -> 12 us at 200 P3, 64 nodes.
+// ---------------------------------------------------------------------------
+template <int N, int NT, bool WIDE = false>
+__global__ void __launch_bounds__(NT)
+k_bounds1d_f64(const double* __restrict__ w, const double* __restrict__ wf, MeshDev m, Phys ph,
+               double* __restrict__ bnd, DevFlags* flags)
+{
+    constexpr int NST = WIDE ? 3 * N : N + 4;
+    __shared__ Bounds1dSmem<NST, NT> sm;
+    const int e = blockIdx.x;
+    if (threadIdx.x < 32) {
+        for (int idx = threadIdx.x; idx < NST * 3; idx += 32) {
+            const int v = idx / NST, r = idx % NST;
+            double val;
+            if (WIDE) val = kbl_wide1d<N>(w, m, e, r, v);
+            else if (r < N) val = w[((size_t)v * m.E + e) * N + r];
+            else if (r < N + 2) val = wf[((size_t)v * m.E + e) * 2 + (r - N)];
+            else val = kbl_exterior<1, N>(wf, m, e, r - N - 2, v);
+            sm.S[r][v] = val;
+        }
+        __syncwarp();
+    }
+    bounds1d_core<NST, NT>(sm, m.E, e, ph, bnd, flags);
+}
+
+// ---------------------------------------------------------------------------
+// 1D, FP32: one block per element, one thread per velocity node (strided), direct evaluation of every
+// Maxwellian.
 // ---------------------------------------------------------------------------
 constexpr int NT1 = 128;
 
-template <int N, bool F32, bool WIDE = false>
+template <int N, bool WIDE = false>
 __global__ void __launch_bounds__(NT1)
-k_bounds1d(const double* __restrict__ w, const double* __restrict__ wf, MeshDev m, Phys ph,
-           double* __restrict__ bnd, DevFlags* flags)
+k_bounds1d_f32(const double* __restrict__ w, const double* __restrict__ wf, MeshDev m, Phys ph,
+               double* __restrict__ bnd, DevFlags* flags)
 {
     constexpr int NS = N, NFP = 2, NST = WIDE ? 3 * NS : NS + 2 * NFP, NV = 3;
     constexpr int NW = NT1 / 32;
@@ -132,71 +160,43 @@ k_bounds1d(const double* __restrict__ w, const double* __restrict__ wf, MeshDev 
     }
     __syncthreads();
     const double lo = sbox[0], h = (sbox[1] - sbox[0]) / (NU - 1);
-    if (!F32) {
-        double acc[8];
+    const double c = 0.5 * (sbox[0] + sbox[1]);
+    float Ur[NST], kx[NST], A[NST], C[NST];
 #pragma unroll
-        for (int k = 0; k < 8; k++) acc[k] = 0.0;
-        for (int j = tid; j < NU; j += NT1) {
-            const double u = lo + j * h;
-            const double M = kbl_qweight(ph, j, NU) * h;
-            double Tl = DBL_MAX, Th = 0.0, Il = DBL_MAX, Ih = 0.0;
+    for (int i = 0; i < NST; i++) {
+        Ur[i] = (float)(sP[i].U[0] - c);
+        kx[i] = (float)(1.4426950408889634 / (2.0 * sP[i].th));
+        A[i] = (float)sP[i].A;
+        C[i] = (float)sP[i].C;
+    }
+    float acc[8];
 #pragma unroll
-            for (int i = 0; i < NST; i++) {
-                const double d = u - sP[i].U[0];
-                const double g = sP[i].A * exp(-(d * d) / (2.0 * sP[i].th));
-                const double cg = sP[i].C * g;
-                Tl = fmin(Tl, g); Th = fmax(Th, g);
-                Il = fmin(Il, cg); Ih = fmax(Ih, cg);
-            }
-            acc[0] += M * Tl;
-            acc[1] += M * Th;
-            if (u < 0.0) { acc[2] += M * Th * u; acc[3] += M * Tl * u; }
-            else { acc[4] += M * Tl * u; acc[5] += M * Th * u; }
-            const double ke = 0.5 * u * u;
-            acc[6] += M * (Tl * ke + Il);
-            acc[7] += M * (Th * ke + Ih);
-        }
-        block_sum_f64<8, NT1>(acc, sred);
-        if (tid == 0) finalize_bounds<1>(acc, 1.0, ph, bnd, m.E, e);
-    } else {
-        const double c = 0.5 * (sbox[0] + sbox[1]);
-        float Ur[NST], kx[NST], A[NST], C[NST];
+    for (int k = 0; k < 8; k++) acc[k] = 0.0f;
+    for (int j = tid; j < NU; j += NT1) {
+        const double ud = lo + j * h;
+        const float u = (float)ud, ur = (float)(ud - c);
+        const float q = (float)kbl_qweight(ph, j, NU);
+        float Tl = FLT_MAX, Th = 0.0f, Il = FLT_MAX, Ih = 0.0f;
 #pragma unroll
         for (int i = 0; i < NST; i++) {
-            Ur[i] = (float)(sP[i].U[0] - c);
-            kx[i] = (float)(1.4426950408889634 / (2.0 * sP[i].th));
-            A[i] = (float)sP[i].A;
-            C[i] = (float)sP[i].C;
+            const float d = ur - Ur[i];
+            const float g = A[i] * fast_exp2(-(d * d) * kx[i]);
+            const float cg = C[i] * g;
+            Tl = fminf(Tl, g); Th = fmaxf(Th, g);
+            Il = fminf(Il, cg); Ih = fmaxf(Ih, cg);
         }
-        float acc[8];
-#pragma unroll
-        for (int k = 0; k < 8; k++) acc[k] = 0.0f;
-        for (int j = tid; j < NU; j += NT1) {
-            const double ud = lo + j * h;
-            const float u = (float)ud, ur = (float)(ud - c);
-            const float q = (float)kbl_qweight(ph, j, NU);
-            float Tl = FLT_MAX, Th = 0.0f, Il = FLT_MAX, Ih = 0.0f;
-#pragma unroll
-            for (int i = 0; i < NST; i++) {
-                const float d = ur - Ur[i];
-                const float g = A[i] * fast_exp2(-(d * d) * kx[i]);
-                const float cg = C[i] * g;
-                Tl = fminf(Tl, g); Th = fmaxf(Th, g);
-                Il = fminf(Il, cg); Ih = fmaxf(Ih, cg);
-            }
-            Tl *= q; Th *= q; Il *= q; Ih *= q;
-            acc[0] += Tl;
-            acc[1] += Th;
-            if (u < 0.0f) { acc[2] += Th * u; acc[3] += Tl * u; }
-            else { acc[4] += Tl * u; acc[5] += Th * u; }
-            const float ke = (float)(0.5 * ud * ud);
-            acc[6] += Tl * ke + Il;
-            acc[7] += Th * ke + Ih;
-        }
-        double tot[8];
-        block_sum_f32c<8, NT1>(acc, tot, reinterpret_cast<float*>(sred));
-        if (tid == 0) finalize_bounds<1>(tot, h, ph, bnd, m.E, e);
+        Tl *= q; Th *= q; Il *= q; Ih *= q;
+        acc[0] += Tl;
+        acc[1] += Th;
+        if (u < 0.0f) { acc[2] += Th * u; acc[3] += Tl * u; }
+        else { acc[4] += Tl * u; acc[5] += Th * u; }
+        const float ke = (float)(0.5 * ud * ud);
+        acc[6] += Tl * ke + Il;
+        acc[7] += Th * ke + Ih;
     }
+    double tot[8];
+    block_sum_f32c<8, NT1>(acc, tot, reinterpret_cast<float*>(sred));
+    if (tid == 0) finalize_bounds<1>(tot, h, ph, bnd, m.E, e);
 }
 
 // ---------------------------------------------------------------------------
@@ -242,12 +242,18 @@ int run_bounds(const kbl_ctx* c, const double* w, const double* wf, double* bnd,
 {
     if (c->E == 0) return 0;
     if (DIM == 1) {
-        const bool f32 = c->cfg.precision == KBL_FP32_MIXED, wide = c->cfg.stencil == 1;
+        const bool wide = c->cfg.stencil == 1;
         const MeshDev m = mesh_of(c);
-        if (f32 && wide) k_bounds1d<N, true, true><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
-        else if (f32) k_bounds1d<N, true><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
-        else if (wide) k_bounds1d<N, false, true><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
-        else k_bounds1d<N, false><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+        if (c->cfg.precision == KBL_FP32_MIXED) {
+            if (wide) k_bounds1d_f32<N, true><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+            else k_bounds1d_f32<N><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+        } else if (c->cfg.nu[0] <= 64) {   // a thread per node where that many suffice
+            if (wide) k_bounds1d_f64<N, 64, true><<<c->E, 64, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+            else k_bounds1d_f64<N, 64><<<c->E, 64, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+        } else {
+            if (wide) k_bounds1d_f64<N, 256, true><<<c->E, 256, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+            else k_bounds1d_f64<N, 256><<<c->E, 256, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+        }
         return 1;
     }
     if (c->cfg.precision != KBL_FP32_MIXED) {

@@ -1037,6 +1037,257 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
     }
 }
 
+// ---------------------------------------------------------------------------
+// 1D, full precision: every Maxwellian of a node as three floats (exp2_pair on fixed-point
+// exponents), the envelopes by comparing their leading two, the sums in FP64
+// ---------------------------------------------------------------------------
+// Per-state constants: as PairState, the step in units of 2^-(58 + floor(log2 nu)).
+struct LineState {
+    long long z, dz;
+    Triple A, C;
+};
+
+// The larger (UP) or smaller of best and x, decided on the leading two floats.
+template <bool UP>
+__device__ __forceinline__ void triple_extreme(Triple& best, const Triple& x)
+{
+    const float d = __fadd_rn(__fsub_rn(x.h, best.h), __fsub_rn(x.l, best.l));
+    if (UP ? d > 0.0f : d < 0.0f) best = x;
+}
+__device__ __forceinline__ double triple_value(const Triple& a)
+{
+    return widen_fast(a.h) + (widen_fast(a.l) + widen_fast(a.r));
+}
+
+// Add node u's terms to the raw sums of finalize_bounds<1>.
+__device__ __forceinline__ void line_moments(double (&acc)[8], double u, double Tl, double Th, double Il, double Ih)
+{
+    acc[0] += Tl;
+    acc[1] += Th;
+    if (u < 0.0) { acc[2] = fma(Th, u, acc[2]); acc[3] = fma(Tl, u, acc[3]); }
+    else { acc[4] = fma(Tl, u, acc[4]); acc[5] = fma(Th, u, acc[5]); }
+    const double ke = 0.5 * u * u;
+    acc[6] += fma(Tl, ke, Il);
+    acc[7] += fma(Th, ke, Ih);
+}
+
+// Raw sums of one thread's nodes by FP64 exponentials: stencils out of the floats' range.
+struct LineSums {
+    double v[8];
+};
+template <int NST>
+__device__ __noinline__ LineSums bounds1d_f64_nodes(const StatePrim* sP, const Phys& ph, double lo, double h, int tid,
+                                                    int nt)
+{
+    LineSums s;
+#pragma unroll
+    for (int k = 0; k < 8; k++) s.v[k] = 0.0;
+    for (int j = tid; j < ph.nu[0]; j += nt) {
+        const double u = lo + j * h, q = kbl_qweight(ph, j, ph.nu[0]);
+        double Tl = DBL_MAX, Th = 0.0, Il = DBL_MAX, Ih = 0.0;
+        for (int i = 0; i < NST; i++) {
+            const double d = u - sP[i].U[0];
+            const double g = sP[i].A * exp(-(d * d) / (2.0 * sP[i].th));
+            const double cg = sP[i].C * g;
+            Tl = fmin(Tl, g); Th = fmax(Th, g);
+            Il = fmin(Il, cg); Ih = fmax(Ih, cg);
+        }
+        line_moments(s.v, u, q * Tl, q * Th, q * Il, q * Ih);
+    }
+    return s;
+}
+
+template <int NST, int NT>
+struct Bounds1dSmem {
+    double S[NST][3];
+    LineState P[NST];
+    StatePrim G[NST];      // the FP64 path's
+    float2 kT[128];        // kbl_exp2_knots
+    int kF[128];
+    double lo, h, c;       // box end, spacing and node (nu - 1) / 2
+    int eA, eU;            // exponents taken out of A and of the velocities
+    double red[NT / 32][8];
+};
+
+// Bounds of element e, one block of NT threads, sm.S filled by the threads of warp 0 (or with a
+// barrier after).
+template <int NST, int NT>
+__device__ __forceinline__ void bounds1d_core(Bounds1dSmem<NST, NT>& sm, int E, int e, const Phys& ph,
+                                              double* __restrict__ bnd, DevFlags* flags)
+{
+    static_assert(NST <= 32, "the states of one warp");
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nu = ph.nu[0], jc = (nu - 1) / 2;
+    const int sh = 31 - __clz(nu);
+    for (int k = tid; k < 128; k += NT) {
+        const Exp2Knot q = kbl_exp2_knots[k];
+        sm.kT[k] = make_float2(__uint_as_float(q.hi), __uint_as_float(q.lo));
+        sm.kF[k] = q.f;
+    }
+    int bad = 0, out_of_range = 0;
+    if (wid == 0) {   // the states, one lane each; the other warps wait
+        double th = 1.0, rs = 1.0, U = 0.0, rho = 1.0;
+        long long klo = 0x7fffffffffffffffll, khi = -0x7fffffffffffffffll;
+        if (lane < NST) {
+            rho = sm.S[lane][0];
+            const double mx = sm.S[lane][1], En = sm.S[lane][2];
+            if (exponent_ok(rho) && exponent_ok(En)) {
+                const double inv = 1.0 / rho;
+                const double P = (ph.gamma - 1.0) * (En - quotient_of(0.5 * (mx * mx), rho, inv));
+                bad = !(P > 0.0);
+                th = quotient_of(P, rho, inv);
+                U = quotient_of(mx, rho, inv);
+                out_of_range = !exponent_ok(th);
+            } else {
+                bad = !(rho > 0.0) || !(kbl_pressure<1>(sm.S[lane], ph.gamma - 1.0) > 0.0);
+                out_of_range = 1;
+            }
+            rs = rsqrt(th);
+            double sq = th * rs;
+            sq = fma(fma(-sq, sq, th), 0.5 * rs, sq);
+            klo = key64(fma(-ph.k, sq, U));
+            khi = key64(fma(ph.k, sq, U));
+        }
+        const double A = rho * rs;                    // 1 / sqrt(2 pi) is in the exponents
+        int kA = lane < NST ? __double2hiint(A) : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            klo = min(klo, __shfl_xor_sync(0xffffffffu, klo, o));
+            khi = max(khi, __shfl_xor_sync(0xffffffffu, khi, o));
+            kA = max(kA, __shfl_xor_sync(0xffffffffu, kA, o));
+        }
+        const double la = unkey64(klo), lb = unkey64(khi), h = (lb - la) / (nu - 1), c = fma((double)jc, h, la);
+        const int eA = (kA >> 20) - 1023;
+        const int eU = (max(__double2hiint(la) & 0x7fffffff, __double2hiint(lb) & 0x7fffffff) >> 20) - 1022;
+        if (abs(eA) > 900 || abs(eU) > 450) out_of_range = 1;
+        const double sA = pow2_f64(abs(eA) > 900 ? 0 : -eA), sU = pow2_f64(abs(eU) > 450 ? 0 : -eU);
+        const double rl = rsqrt_rest(th, rs);
+        Triple At = split_f32(A * sA);
+        At.r += (float)(fma(rho, rs, -A) * sA + rho * rl * sA);
+        const Triple Ct = split_f32(ph.half_delta1 * th * (sU * sU));
+        const double kh = 0.8493218002880191 * rs;
+        const double kl = fma(0.8493218002880191, rs, -kh) + fma(-2.5959464104597403e-17, rs, 0.8493218002880191 * rl);
+        const double dc = c - U, zh = dc * kh, dh = h * kh;
+        const double zl = fma(dc, kl, fma(dc, kh, -zh)), dl = fma(h, kl, fma(h, kh, -dh));
+        const double up = pow2_f64(sh);
+        if (lane < NST) {
+            sm.P[lane].z = fixed58(zh) + fixed58(zl);
+            sm.P[lane].dz = fixed58(dh * up) + fixed58(dl * up);   // below 31 by the range test
+            sm.P[lane].A = At;
+            sm.P[lane].C = Ct;
+            const float tm = fabsf(f32_trunc(zh)) + f32_trunc(dh) * (float)(nu / 2 + 1);
+            if (!(tm < 15.5f) || !(At.h >= 0x1p-60f) || !(Ct.h == 0.0f || (Ct.h >= 0x1p-30f && Ct.h < 0x1p60f)))
+                out_of_range = 1;
+        }
+        if (lane == 0) {
+            sm.lo = la;
+            sm.h = h;
+            sm.c = c;
+            sm.eA = eA;
+            sm.eU = eU;
+        }
+    }
+    if (__syncthreads_or(bad)) {
+        if (tid == 0) {
+            write_nan(bnd, E, e, 3);
+            atomicOr(&flags->nonphysical, 1);
+        }
+        return;
+    }
+    bool pairs = !__syncthreads_or(out_of_range);
+    for (;;) {
+        double acc[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) acc[k] = 0.0;
+        const double lo = sm.lo, h = sm.h;
+        if (pairs) {
+            const double sU = pow2_f64(-sm.eU);
+            for (int j = tid; j < nu; j += NT) {
+                Triple Tl, Th, Il, Ih;
+                const long long k = (long long)(j - jc) << (63 - sh);
+#pragma unroll 1
+                for (int i = 0; i < NST; i += 2) {
+                    const LineState& s0 = sm.P[i];
+                    const LineState& s1 = sm.P[i + 1 < NST ? i + 1 : i];
+                    auto exponent = [&](const LineState& s) {
+                        const long long z = s.z + 2 * __mul64hi(s.dz, k);
+                        const unsigned long long z4 = 4ull * (unsigned long long)(z < 0 ? -z : z);
+                        return (long long)((__umul64hi(z4, z4) + 1ull) >> 1) + 47765107922663390ll;   // log2(2 pi) / 2
+                    };
+                    int n0, n1;
+                    Triple2 y = exp2_pair(exponent(s0), exponent(s1), sm.kT, sm.kF, n0, n1);
+                    const float2 sc = make_float2(n0 < 120 ? __uint_as_float((unsigned)(127 - n0) << 23) : 0.0f,
+                                                  n1 < 120 ? __uint_as_float((unsigned)(127 - n1) << 23) : 0.0f);
+                    y = triple_mul(y, make_float2(s0.A.h, s1.A.h), make_float2(s0.A.l, s1.A.l),
+                                   make_float2(s0.A.r, s1.A.r));
+                    const Triple2 c = triple_mul(y, make_float2(s0.C.h, s1.C.h), make_float2(s0.C.l, s1.C.l),
+                                                 make_float2(s0.C.r, s1.C.r));
+                    const Triple T0 = {y.h.x * sc.x, y.l.x * sc.x, y.r.x * sc.x}, T1 = {y.h.y * sc.y, y.l.y * sc.y, y.r.y * sc.y};
+                    const Triple I0 = {c.h.x * sc.x, c.l.x * sc.x, c.r.x * sc.x}, I1 = {c.h.y * sc.y, c.l.y * sc.y, c.r.y * sc.y};
+                    if (i == 0) { Tl = Th = T0; Il = Ih = I0; }
+                    else {
+                        triple_extreme<false>(Tl, T0); triple_extreme<true>(Th, T0);
+                        triple_extreme<false>(Il, I0); triple_extreme<true>(Ih, I0);
+                    }
+                    triple_extreme<false>(Tl, T1); triple_extreme<true>(Th, T1);
+                    triple_extreme<false>(Il, I1); triple_extreme<true>(Ih, I1);
+                }
+                const double u = (lo + j * h) * sU, q = kbl_qweight(ph, j, nu);
+                line_moments(acc, u, q * triple_value(Tl), q * triple_value(Th), q * triple_value(Il), q * triple_value(Ih));
+            }
+        } else {
+            if (tid < NST) prim_of<1>(sm.S[tid], ph, sm.G[tid]);
+            __syncthreads();
+            if (tid == 0) {   // the box of the states as they are
+                double a = sm.G[0].U[0] - ph.k * sm.G[0].sq, b = sm.G[0].U[0] + ph.k * sm.G[0].sq;
+                for (int i = 1; i < NST; i++) {
+                    a = fmin(a, sm.G[i].U[0] - ph.k * sm.G[i].sq);
+                    b = fmax(b, sm.G[i].U[0] + ph.k * sm.G[i].sq);
+                }
+                sm.lo = a;
+                sm.h = (b - a) / (nu - 1);
+            }
+            __syncthreads();
+            const LineSums s = bounds1d_f64_nodes<NST>(sm.G, ph, sm.lo, sm.h, tid, NT);
+#pragma unroll
+            for (int k = 0; k < 8; k++) acc[k] = s.v[k];
+        }
+        // warp reduce-scatter (lane 4 k holds sum k), then the warps
+#pragma unroll
+        for (int step = 0; step < 3; step++) {
+            const int off = 16 >> step, n = 4 >> step;
+            const bool up = lane & off;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (k >= n) break;
+                const double keep = up ? acc[n + k] : acc[k], send = up ? acc[k] : acc[n + k];
+                acc[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
+        }
+#pragma unroll
+        for (int off = 2; off > 0; off >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], off);
+        if ((lane & 3) == 0) sm.red[wid][lane >> 2] = acc[0];
+        __syncthreads();
+        int redo = 0;
+        if (tid < 8) {
+            double s = sum_warps<NT / 32>(sm.red, tid);
+            if (pairs) {
+                if (tid == 0 && !(s >= 0x1p-40)) redo = 1;   // sums of floats that may have underflowed
+                s *= pow2_f64(sm.eA) * (tid < 2 ? 1.0 : tid < 6 ? pow2_f64(sm.eU) : pow2_f64(2 * sm.eU));
+            }
+            // times h and the relaxation of the sum's envelope, rounded once
+            const double r = (0xa6 >> tid) & 1 ? ph.rel_hi : ph.rel_lo, p = s * sm.h;
+            s = fma(r, p, r * fma(s, sm.h, -p));
+            // raw sums: Tlo, Thi, n_hi, n_lo, p_lo, p_hi, E_lo, E_hi; lane 2 + 4 and 3 + 5 make the momentum
+            const double t = __shfl_down_sync(0xffu, s, 2);
+            if (tid == 0 && s < ph.rho_floor) s = ph.rho_floor;
+            if (tid == 2 || tid == 3) s += t;
+            if (tid < 4 || tid > 5) bnd[((size_t)(tid & 1) * 3 + (tid < 2 ? 0 : tid < 4 ? 1 : 2)) * E + e] = s;
+        }
+        if (!__syncthreads_or(redo)) break;
+        pairs = false;
+    }
+}
+
 // The block's dynamic shared memory as one object.
 template <typename SM>
 __device__ __forceinline__ SM& kbl_dyn_smem()

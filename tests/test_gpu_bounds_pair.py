@@ -86,3 +86,49 @@ def test_fast_streams(orc):
         _check(orc, S, 32)
     S = inputs.random_states(np.random.default_rng(8), 40, 2, vel=(50.0, 60.0)).reshape(5, 8, 4)
     _check(orc, S, 32)
+
+
+def _line(orc, w, mesh, p, nu, tol=TOL, **kw):
+    from paper_2407_20966_gb300 import kbl
+    E = mesh.n_elem
+    ctx = kbl.Context(dim=1, p=p, nu=(nu,), precision=kbl.FP64, **kw)
+    ctx.mesh_upload(mesh.nbr, mesh.h, mesh.bc)
+    cfg = orc.Config(dim=1, p=p, nu=(nu,), **kw)
+    wf, bnd = zeros_dev(3, E, 2), zeros_dev(2, 3, E)
+    wd = to_dev(w)
+    ctx.traces(wd, wf)
+    ctx.bounds(wd, wf, bnd)
+    ctx.check()
+    om = orc.Mesh(mesh.nbr, mesh.h, mesh.bc)
+    ref = orc.bounds(cfg, om, w, wf.cpu().numpy())
+    got = bnd.cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        err = np.where(got == ref, 0.0, bounds_error(got, ref)).max()
+    assert err < tol, err
+
+
+def _line_field(p, n=23, seed=0):
+    mesh = inputs.mesh_1d(n, 0.0, 1.0, periodic=True)
+    xi = np.polynomial.legendre.leggauss(p + 1)[0]
+    return mesh, inputs.random_discontinuous_field(np.random.default_rng(seed), mesh, xi)
+
+
+@pytest.mark.parametrize("p,nu,kw", [
+    (1, 2, {}), (2, 3, {}), (3, 5, {}), (4, 63, {}), (3, 64, {}), (5, 65, dict(quadrature=1)), (3, 255, {}),
+    (2, 257, dict(quadrature=1, k=8.0)), (4, 2048, dict(k=8.0, r_fac=0.0)), (1, 4096, {}),
+    (3, 64, dict(stencil=1)), (5, 100, dict(stencil=1)), (3, 64, dict(gamma=3.0))])
+def test_line_nodes_and_stencils(orc, p, nu, kw):
+    """1D: node counts around the block sizes, both stencils, delta = 0."""
+    mesh, w = _line_field(p)
+    _line(orc, w, mesh, p, nu, **kw)
+
+
+@pytest.mark.parametrize("ratio", [3.0, 30.0, 1e5])
+def test_line_jumps_and_scales(orc, ratio):
+    """1D jumps that leave the floats' range inside the box, and scaled states."""
+    mesh, ic = inputs.riemann_1d(12, (1.0, 0.3, ratio), (0.5, -0.2, 1.0), 0.0, 1.0, 0.5)
+    w = inputs.nodal_field(mesh, np.polynomial.legendre.leggauss(4)[0], ic)
+    _line(orc, w, mesh, 3, 64)
+    s = np.array([1e-40, 1e-40 * 1e30, 1e-40 * 1e60])
+    mesh.bc = mesh.bc * s
+    _line(orc, w * s[:, None, None], mesh, 3, 100, rho_floor=0.0)
