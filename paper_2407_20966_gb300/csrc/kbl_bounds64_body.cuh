@@ -319,12 +319,16 @@ __device__ __forceinline__ void bounds2d_f64_core(Bounds2dF64Smem<NST, NX>& sm, 
 //   moments      the nodes' values in error-free FP32 sums along rows and columns, those in FP64;
 //                the quadrature weights are in the tables already
 //
-// Measured at 128^2 P3, 32^2 grid: 0.95 ms per launch (1.08 ms with the moments node by node in FP64 and
-// the states' constants in two passes over shared memory), 6.52 ms for the FP64 kernel above (86% of
-// the FP64 pipe); 33^2 Romberg grid (46 x 27 P4): 0.24 ms on a 40-node tile, 2.77 ms on the FP64
-// kernel's 64.
+// Measured at 128^2 P3, 32^2 grid: 0.87 ms per launch; 0.95 with the y table's values stored twice (a
+// 128-bit shared load takes four wavefronts however many lanes share its addresses, and the passes
+// wait on them: 6.9k of 19k clocks per element), 1.08 with the moments node by node in FP64 and the
+// states' constants in two passes over shared memory, 6.52 for the FP64 kernel above (86% of the FP64
+// pipe).  33^2 Romberg grid (46 x 27 P4): 0.21 ms on a 40-node tile, 2.77 ms on the FP64 kernel's 64.
+// Five blocks per SM (96 registers): 0.90 ms against 0.85 (kernel alone) at 48 states, 0.54 against
+// 0.57 at 24.
 // What bounds it: per (state, node) 14 FP32 products/FMAs (packed two to an instruction, two
-// neighbouring x nodes) and four three-input min/max, 7 + 4 issue slots.
+// neighbouring x nodes) and four three-input min/max, 7 + 4 issue slots: about half the launch; the
+// states' FP64 chains, tables and sums the other half.
 //
 // Elements outside the range of the pairs (a state more than 2^240 below its peak inside the box,
 // constants beyond +-2^60 of the largest, a lower density sum below 2^-40 of the largest state's)
@@ -568,7 +572,7 @@ struct Bounds2dPairSmem {
     union __align__(16) {
         struct {
             float x[NSTP][4][NX];     // a_hi, a_lo, c_hi, c_lo
-            float4 y[NSTP][NX];       // b_hi twice, b_lo twice
+            float y[NSTP][2][NX];     // b_hi, b_lo
         } tab;
         F64Tables<NST, NX, NW> gen;   // an element out of the pairs' range
     } u;
@@ -846,8 +850,8 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
                 *(float2*)&sm.u.tab.x[i][3][j] = l;
             } else {
                 triple_store(y, sc, ca, h, l);
-                sm.u.tab.y[i][j] = make_float4(h.x, h.x, l.x, l.x);
-                sm.u.tab.y[i][j + 1] = make_float4(h.y, h.y, l.y, l.y);
+                *(float2*)&sm.u.tab.y[i][0][j] = h;
+                *(float2*)&sm.u.tab.y[i][1][j] = l;
             }
             dt += dd;
             t = t1 + dt;
@@ -878,10 +882,10 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
             const float2 A1[2] = {make_float2(a1.x, a1.y), make_float2(a1.z, a1.w)};
             const float2 C0[2] = {make_float2(c0.x, c0.y), make_float2(c0.z, c0.w)};
             const float2 C1[2] = {make_float2(c1.x, c1.y), make_float2(c1.z, c1.w)};
+            const float2 b0 = *(const float2*)&sm.u.tab.y[i][0][ty * TY], b1 = *(const float2*)&sm.u.tab.y[i + 1][0][ty * TY];
 #pragma unroll
             for (int b = 0; b < TY; b++) {
-                const float2 y0 = *(const float2*)&sm.u.tab.y[i][ty * TY + b];
-                const float2 y1 = *(const float2*)&sm.u.tab.y[i + 1][ty * TY + b];
+                const float2 y0 = f2dup(b ? b0.y : b0.x), y1 = f2dup(b ? b1.y : b1.x);
 #pragma unroll
                 for (int p = 0; p < 2; p++) {
                     const float2 g0 = __fmul2_rn(A0[p], y0), g1 = __fmul2_rn(A1[p], y1);
@@ -918,11 +922,15 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
                     X[s][k][0] = make_float2(v.x, v.y);
                     X[s][k][1] = make_float2(v.z, v.w);
                 }
+            float2 Y[2][2];      // [state][b_hi, b_lo] of both y nodes
+#pragma unroll
+            for (int s = 0; s < 2; s++)
+#pragma unroll
+                for (int k = 0; k < 2; k++) Y[s][k] = *(const float2*)&sm.u.tab.y[i + s][k][ty * TY];
 #pragma unroll
             for (int b = 0; b < TY; b++) {
-                const float4 v0 = sm.u.tab.y[i][ty * TY + b], v1 = sm.u.tab.y[i + 1][ty * TY + b];
-                const float2 bh0 = make_float2(v0.x, v0.y), bl0 = make_float2(v0.z, v0.w);
-                const float2 bh1 = make_float2(v1.x, v1.y), bl1 = make_float2(v1.z, v1.w);
+                const float2 bh0 = f2dup(b ? Y[0][0].y : Y[0][0].x), bl0 = f2dup(b ? Y[0][1].y : Y[0][1].x);
+                const float2 bh1 = f2dup(b ? Y[1][0].y : Y[1][0].x), bl1 = f2dup(b ? Y[1][1].y : Y[1][1].x);
 #pragma unroll
                 for (int p = 0; p < 2; p++) {
                     // a b - M of both states
