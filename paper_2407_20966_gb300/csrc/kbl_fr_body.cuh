@@ -68,7 +68,9 @@ __device__ __forceinline__ void rhs_block(RhsSmem<DIM, N, T, EPB>& sm, int NT, c
     const T gamma = from_f64<T>(gamma_d), gm1 = F32 ? gamma - T(1) : from_f64<T>(gamma_d - 1.0);
     // the first face point of this thread: its interior and exterior values are loaded now, so
     // that their latency (the exterior one behind the neighbour index) overlaps step 1
-    double pi[NV], pe[NV];
+    // (minus and plus side of the axis: a flux call per side would run twice in every warp, whose lanes
+    // hold faces of both sides)
+    double pl[NV], pr[NV];
     bool pre = false;
     {
         const int ell = tid / NFP, fp = tid % NFP, ee = e0 + ell;
@@ -76,8 +78,10 @@ __device__ __forceinline__ void rhs_block(RhsSmem<DIM, N, T, EPB>& sm, int NT, c
             pre = true;
 #pragma unroll
             for (int v = 0; v < NV; v++) {
-                pi[v] = wf[((size_t)v * m.E + ee) * NFP + fp];
-                pe[v] = kbl_exterior<DIM, N>(wf, m, ee, fp, v);
+                const double qi = wf[((size_t)v * m.E + ee) * NFP + fp], qe = kbl_exterior<DIM, N>(wf, m, ee, fp, v);
+                const bool plus = (fp / NFPF) & 1;
+                pl[v] = plus ? qi : qe;
+                pr[v] = plus ? qe : qi;
             }
         }
     }
@@ -99,30 +103,25 @@ __device__ __forceinline__ void rhs_block(RhsSmem<DIM, N, T, EPB>& sm, int NT, c
         const int ee = e0 + ell;
         if (ee >= m.E || ell >= nmax) continue;
         const int f = fp / NFPF, k = fp % NFPF, dir = f >> 1, side = f & 1;
-        T qi[NV], qe[NV], Fc[NV];
+        T ql[NV], qr[NV], Fc[NV];
         if (pre && t == tid) {
 #pragma unroll
             for (int v = 0; v < NV; v++) {
-                qi[v] = from_f64<T>(pi[v]);
-                qe[v] = from_f64<T>(pe[v]);
+                ql[v] = from_f64<T>(pl[v]);
+                qr[v] = from_f64<T>(pr[v]);
             }
         } else {
 #pragma unroll
             for (int v = 0; v < NV; v++) {
-                qi[v] = from_f64<T>(wf[((size_t)v * m.E + ee) * NFP + fp]);
-                qe[v] = from_f64<T>(kbl_exterior<DIM, N>(wf, m, ee, fp, v));
+                const T qi = from_f64<T>(wf[((size_t)v * m.E + ee) * NFP + fp]);
+                const T qe = from_f64<T>(kbl_exterior<DIM, N>(wf, m, ee, fp, v));
+                ql[v] = side ? qi : qe;
+                qr[v] = side ? qe : qi;
             }
         }
-        if (flux == 1) {
-            if (side == 0) kbl_hllc<DIM, T>(qe, qi, dir, gamma, Fc);
-            else kbl_hllc<DIM, T>(qi, qe, dir, gamma, Fc);
-        } else if (flux == 2) {
-            if (side == 0) kbl_hll<DIM, T>(qe, qi, dir, gamma, Fc);
-            else kbl_hll<DIM, T>(qi, qe, dir, gamma, Fc);
-        } else {
-            if (side == 0) kbl_rusanov<DIM, T>(qe, qi, dir, gamma, Fc);
-            else kbl_rusanov<DIM, T>(qi, qe, dir, gamma, Fc);
-        }
+        if (flux == 1) kbl_hllc<DIM, T>(ql, qr, dir, gamma, Fc);
+        else if (flux == 2) kbl_hll<DIM, T>(ql, qr, dir, gamma, Fc);
+        else kbl_rusanov<DIM, T>(ql, qr, dir, gamma, Fc);
         const T* l = side ? slp : slm;
 #pragma unroll
         for (int v = 0; v < NV; v++) {
