@@ -90,6 +90,7 @@ k_rhs_vjp(const double* __restrict__ w, const double* __restrict__ wf, const dou
         const int f = fp / N, k = fp % N, dir = f >> 1, side = f & 1;
         const double s = dir ? 2.0 / m.h[ee * 2 + 1] : 2.0 / m.h[ee * 2 + 0];
         double Jb[NV];
+#pragma unroll
         for (int v = 0; v < NV; v++) {
             double acc = 0.0;
             for (int a = 0; a < N; a++)
@@ -97,19 +98,29 @@ k_rhs_vjp(const double* __restrict__ w, const double* __restrict__ wf, const dou
             Jb[v] = -s * acc;
             sJb[ell][fp][v] = Jb[v];
         }
-        // J = Fc(q_left, q_right) - F^D: the common flux
-        double qi[NV], qe[NV], qib[NV] = {0, 0, 0, 0}, qeb[NV] = {0, 0, 0, 0};
+        // J = Fc(q_left, q_right) - F^D: the common flux, with the states on the minus and the plus side
+        // selected by value and, on y faces, the momenta exchanged, so that the warp's lanes, which hold
+        // faces of both axes and sides, run one flux adjoint and not four
+        const int vx = 1 + dir, vy = 2 - dir;   // momentum along the axis and across it
+        double ql[NV], qr[NV], Fb[NV], qlb[NV] = {0, 0, 0, 0}, qrb[NV] = {0, 0, 0, 0};
         const int nb = m.nbr[ee * 4 + f];
-        for (int v = 0; v < NV; v++) {
-            qi[v] = wf[((size_t)v * m.E + ee) * NFP + fp];
-            qe[v] = nb >= 0 ? wf[((size_t)v * m.E + nb) * NFP + (f ^ 1) * N + k] : m.bc[(-nb - 1) * NV + v];
+#pragma unroll
+        for (int k2 = 0; k2 < NV; k2++) {
+            const int v = k2 == 1 ? vx : k2 == 2 ? vy : k2;
+            const double qi = wf[((size_t)v * m.E + ee) * NFP + fp];
+            const double qe = nb >= 0 ? wf[((size_t)v * m.E + nb) * NFP + (f ^ 1) * N + k] : m.bc[(-nb - 1) * NV + v];
+            ql[k2] = side ? qi : qe;
+            qr[k2] = side ? qe : qi;
+            Fb[k2] = k2 == 1 ? (dir ? Jb[2] : Jb[1]) : k2 == 2 ? (dir ? Jb[1] : Jb[2]) : Jb[k2];
         }
-        if (dir == 0) {
-            if (side == 0) rusanov_vjp<2, 0>(qe, qi, gamma, Jb, qeb, qib);
-            else rusanov_vjp<2, 0>(qi, qe, gamma, Jb, qib, qeb);
-        } else {
-            if (side == 0) rusanov_vjp<2, 1>(qe, qi, gamma, Jb, qeb, qib);
-            else rusanov_vjp<2, 1>(qi, qe, gamma, Jb, qib, qeb);
+        rusanov_vjp<2, 0>(ql, qr, gamma, Fb, qlb, qrb);
+        double qib[NV], qeb[NV];
+#pragma unroll
+        for (int v = 0; v < NV; v++) {
+            const double l = v == 1 ? (dir ? qlb[2] : qlb[1]) : v == 2 ? (dir ? qlb[1] : qlb[2]) : qlb[v];
+            const double r = v == 1 ? (dir ? qrb[2] : qrb[1]) : v == 2 ? (dir ? qrb[1] : qrb[2]) : qrb[v];
+            qib[v] = side ? l : r;
+            qeb[v] = side ? r : l;
         }
         for (int v = 0; v < NV; v++) {
             wfb[((size_t)v * m.E + ee) * NFP + fp] += qib[v];
@@ -146,9 +157,13 @@ k_rhs_vjp(const double* __restrict__ w, const double* __restrict__ wf, const dou
 //      -/+ (bndb . B_j) / (hi - lo);
 //   c) the box ends are min / max over the stencil of U -+ k sqrt(theta) (Eq. 45):
 //      their cotangents go to the winning states.
-// Pass A (per grid point) finds the winners and the envelope cotangents; pass B (per
-// stencil state) re-evaluates only the Maxwellians that won and accumulates (a) and
-// their share of (b).  The grid is processed in chunks of at most 1024 points.
+// Pass A (per grid point) finds the winners and the envelope cotangents; pass B (a warp per
+// stencil state) gathers the points where its state won, 32 at a time, re-evaluates only those
+// Maxwellians and accumulates (a) and their share of (b).  The grid is processed in chunks of at
+// most 1024 points.  Few elements have a cotangent, so a launch lasts as long as one block: with a
+// thread per (state, fifth of the points) every win cost a warp the FP64 body for one lane, and the
+// winners were compared on the FP64 pipe (976 us per launch with an active element, P3, 32^2 grid;
+// 137 us now).
 // ---------------------------------------------------------------------------
 constexpr int NT_BV = 256;
 
@@ -160,10 +175,8 @@ template <int N, int NX>
 struct BvShape {
     static constexpr int NS = N * N, NFP = 4 * N, NST = NS + 2 * NFP;
     static constexpr int NPTS = NX * NX, CHUNK = NPTS < 1024 ? NPTS : 1024;
-    static constexpr int TPN = NT_BV / NST;  // pass-B threads per stencil state
-    // dynamic shared memory: Ex, C Ex, Ey tables, two chunk cotangents, pass-B partials, winners
-    static constexpr size_t SMEM = sizeof(double) * (3 * NST * NX + 2 * CHUNK + (size_t)NST * TPN * 4) +
-                                   4 * CHUNK;
+    // dynamic shared memory: Ex, C Ex, Ey tables, two chunk cotangents, the warps' queues, winners
+    static constexpr size_t SMEM = sizeof(double) * (3 * NST * NX + 2 * CHUNK) + sizeof(int) * 2 * NT_BV + 4 * CHUNK;
 };
 
 template <int N, int NX>
@@ -174,15 +187,15 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
 {
     using SH = BvShape<N, NX>;
     constexpr int NS = SH::NS, NFP = SH::NFP, NST = SH::NST, NV = 4;
-    constexpr int CHUNK = SH::CHUNK, TPN = SH::TPN, NT = NT_BV, NW = NT / 32;
+    constexpr int CHUNK = SH::CHUNK, NT = NT_BV, NW = NT / 32;
     extern __shared__ double dsm[];
     double(*sEx)[NX] = reinterpret_cast<double(*)[NX]>(dsm);
     double(*sExc)[NX] = sEx + NST;
     double(*sEy)[NX] = sExc + NST;
     double* sWTl = dsm + 3 * NST * NX;
     double* sWTh = sWTl + CHUNK;
-    double* sacc = sWTh + CHUNK;                                            // [TPN][NST][4]
-    unsigned char* sidx = reinterpret_cast<unsigned char*>(sacc + NST * TPN * 4);  // [CHUNK][4]
+    int* squeue = reinterpret_cast<int*>(sWTh + CHUNK);                     // [NW][64]
+    unsigned char* sidx = reinterpret_cast<unsigned char*>(squeue + 2 * NT);   // [CHUNK][4]
     __shared__ double sS[NST][NV];
     __shared__ AdjPrim sP[NST];
     __shared__ double snode[NST][4];   // cotangents of (rho at fixed U, theta), U_x, U_y, theta
@@ -190,9 +203,9 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
     __shared__ double sbox[4], sbb[4];
     __shared__ double sB[8];
     __shared__ double sred[NW * 4];
-    __shared__ int sbad;
+    __shared__ int sbad, sbest[4];
 
-    const int e = blockIdx.x, tid = threadIdx.x;
+    const int e = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     // an element whose bounds were not used by the limiter (zero cotangent) adds nothing
     double b0 = 0.0;
     if (tid < 8) {
@@ -230,15 +243,27 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
         if (tid == 0) atomicOr(&flags->nonphysical, 1);
         return;
     }
-    // box (Eq. 45): value and, in pass C, the first state attaining it
-    if (tid < 4) {
-        const int d = tid >> 1, up = tid & 1;
-        double b = up ? sP[0].U[d] + ph.k * sP[0].sq : sP[0].U[d] - ph.k * sP[0].sq;
-        for (int i = 1; i < NST; i++) {
-            const double c = up ? sP[i].U[d] + ph.k * sP[i].sq : sP[i].U[d] - ph.k * sP[i].sq;
-            b = up ? fmax(b, c) : fmin(b, c);
+    // box (Eq. 45): value and, for pass C, the first state attaining it; a warp per end
+    if (wid < 4) {
+        const int d = wid >> 1;
+        const bool up = wid & 1;
+        auto end = [&](int i) { return up ? sP[i].U[d] + ph.k * sP[i].sq : sP[i].U[d] - ph.k * sP[i].sq; };
+        int best = lane < NST ? lane : 0;
+        double b = end(best);
+        for (int i = lane + 32; i < NST; i += 32) {
+            const double v = end(i);
+            if (up ? v > b : v < b) { b = v; best = i; }
         }
-        sbox[tid] = b;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double v = __shfl_xor_sync(0xffffffffu, b, o);
+            const int i = __shfl_xor_sync(0xffffffffu, best, o);
+            if ((up ? v > b : v < b) || (v == b && i < best)) { b = v; best = i; }
+        }
+        if (lane == 0) {
+            sbox[wid] = b;
+            sbest[wid] = best;
+        }
     }
     __syncthreads();
     for (int j = tid; j < 2 * NX; j += NT) {
@@ -273,24 +298,26 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
     const double Lx = sbox[1] - sbox[0], Ly = sbox[3] - sbox[2];
     const double inv_n1 = 1.0 / (NX - 1);
     double bl_x = 0.0, bh_x = 0.0, bl_y = 0.0, bh_y = 0.0;  // box-end cotangents, this thread's share
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
     for (int c0 = 0; c0 < SH::NPTS; c0 += CHUNK) {
         __syncthreads();
         // pass A: one grid point per thread
         for (int jj = tid; jj < CHUNK; jj += NT) {
             const int j = c0 + jj, jx = j % NX, jy = j / NX;
             const double ux = sux[jx], uy = suy[jy], M = swx[jx] * swy[jy];
-            double tl = DBL_MAX, th = -1.0, il = DBL_MAX, ih = -1.0;
+            // compared as bit patterns: all values are >= +0
+            long long tl = __double_as_longlong(DBL_MAX), th = 0, il = tl, ih = 0;
             int itl = 0, ith = 0, iil = 0, iih = 0;
+#pragma unroll 4
             for (int i = 0; i < NST; i++) {
                 const double ey = sEy[i][jy];
-                const double g = sEx[i][jx] * ey, cg = sExc[i][jx] * ey;
+                const long long g = __double_as_longlong(sEx[i][jx] * ey), cg = __double_as_longlong(sExc[i][jx] * ey);
                 if (g < tl) { tl = g; itl = i; }
                 if (g > th) { th = g; ith = i; }
                 if (cg < il) { il = cg; iil = i; }
                 if (cg > ih) { ih = cg; iih = i; }
             }
-            const double Tl = rm * tl, Th = rp * th, Il = rm * il, Ih = rp * ih;
+            const double Tl = rm * __longlong_as_double(tl), Th = rp * __longlong_as_double(th);
+            const double Il = rm * __longlong_as_double(il), Ih = rp * __longlong_as_double(ih);
             const double ke = 0.5 * (ux * ux + uy * uy);
             const double* lb = sB;
             const double* hb = sB + 4;
@@ -318,39 +345,74 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
             bh_y += uby * ty + MM / Ly;
         }
         __syncthreads();
-        // pass B: threads (state i, sub) scan the chunk for the points where state i won
-        if (tid < NST * TPN) {
-            const int i = tid % NST, sub = tid / NST;
+        // pass B: warp wid takes the states wid, wid + NW, ...; the points a state won queue up and run
+        // 32 at a time, in the order of the points
+        int* const q = squeue + 64 * wid;
+        for (int i = wid; i < NST; i += NW) {
             const AdjPrim s = sP[i];
             const double inv_th = 1.0 / s.th;
-            for (int jj = sub; jj < CHUNK; jj += TPN) {
-                const uchar4 win = reinterpret_cast<const uchar4*>(sidx)[jj];
-                const bool wtl = win.x == i, wth = win.y == i, wil = win.z == i, wih = win.w == i;
-                if (!(wtl | wth | wil | wih)) continue;
+            // sums of G g, G g d, G g |d|^2, g wI and G g d t
+            double S0 = 0.0, Sx = 0.0, Sy = 0.0, S2 = 0.0, SI = 0.0, Stx = 0.0, Sty = 0.0;
+            auto add = [&](int entry) {
+                const int jj = entry & 0xffff, win = entry >> 16;
                 const int j = c0 + jj, jx = j % NX, jy = j / NX;
-                const double ux = sux[jx], uy = suy[jy], M = swx[jx] * swy[jy];
                 const double g = sEx[i][jx] * sEy[i][jy];
-                const double wI = (wil ? rm * M * sB[3] : 0.0) + (wih ? rp * M * sB[7] : 0.0);
-                const double G = (wtl ? sWTl[jj] : 0.0) + (wth ? sWTh[jj] : 0.0) + s.C * wI;
-                const double Gg = G * g;
-                const double dx = ux - s.U[0], dy = uy - s.U[1];
-                acc[0] += Gg / s.rho;
-                acc[1] += Gg * dx * inv_th;
-                acc[2] += Gg * dy * inv_th;
-                acc[3] += Gg * (0.5 * (dx * dx + dy * dy) * inv_th * inv_th - inv_th) + 0.5 * delta * g * wI;
-                const double gx = -Gg * dx * inv_th, gy = -Gg * dy * inv_th;
-                const double tx = jx * inv_n1, ty = jy * inv_n1;
-                bl_x += gx * (1.0 - tx);
-                bh_x += gx * tx;
-                bl_y += gy * (1.0 - ty);
-                bh_y += gy * ty;
+                double wI = 0.0, G = 0.0;
+                if (win & 12) {
+                    const double M = swx[jx] * swy[jy];
+                    wI = M * (((win & 4) ? rm * sB[3] : 0.0) + ((win & 8) ? rp * sB[7] : 0.0));
+                    G = s.C * wI;
+                    SI = fma(g, wI, SI);
+                }
+                if (win & 1) G += sWTl[jj];
+                if (win & 2) G += sWTh[jj];
+                const double Gg = G * g, dx = sux[jx] - s.U[0], dy = suy[jy] - s.U[1];
+                const double gx = Gg * dx, gy = Gg * dy;
+                S0 += Gg;
+                Sx += gx;
+                Sy += gy;
+                S2 = fma(gx, dx, fma(gy, dy, S2));
+                Stx = fma(gx, jx * inv_n1, Stx);
+                Sty = fma(gy, jy * inv_n1, Sty);
+            };
+            int cnt = 0, any = 0;
+            for (int base = 0; base < CHUNK; base += 32) {
+                const uchar4 w4 = reinterpret_cast<const uchar4*>(sidx)[base + lane];
+                const int win = (w4.x == i) | (w4.y == i) << 1 | (w4.z == i) << 2 | (w4.w == i) << 3;
+                const unsigned hit = __ballot_sync(0xffffffffu, win != 0);
+                if (!hit) continue;
+                if (win) q[cnt + __popc(hit & ((1u << lane) - 1u))] = (base + lane) | win << 16;
+                cnt += __popc(hit);
+                any = 1;
+                __syncwarp();
+                if (cnt >= 32) {
+                    add(q[lane]);
+                    cnt -= 32;
+                    const int rest = q[32 + lane];
+                    __syncwarp();
+                    q[lane] = rest;
+                    __syncwarp();
+                }
+            }
+            if (!any) continue;
+            if (lane < cnt) add(q[lane]);
+            __syncwarp();
+            bl_x -= inv_th * (Sx - Stx);
+            bh_x -= inv_th * Stx;
+            bl_y -= inv_th * (Sy - Sty);
+            bh_y -= inv_th * Sty;
+            double r[5] = {S0, Sx, Sy, S2, SI};
+#pragma unroll
+            for (int k = 0; k < 5; k++)
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) r[k] += __shfl_xor_sync(0xffffffffu, r[k], o);
+            if (lane == 0) {
+                snode[i][0] += r[0] / s.rho;
+                snode[i][1] += r[1] * inv_th;
+                snode[i][2] += r[2] * inv_th;
+                snode[i][3] += inv_th * (0.5 * inv_th * r[3] - r[0]) + 0.5 * delta * r[4];
             }
         }
-    }
-    if (tid < NST * TPN) {
-        const int i = tid % NST, sub = tid / NST;
-#pragma unroll
-        for (int k = 0; k < 4; k++) sacc[(sub * NST + i) * 4 + k] = acc[k];
     }
     // box-end cotangents: block sum (fixed order)
     double bb[4] = {bl_x, bh_x, bl_y, bh_y};
@@ -367,21 +429,11 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
         for (int q = 0; q < NW; q++) s += sred[q * 4 + tid];
         sbb[tid] = s;
     }
-    for (int i = tid; i < NST; i += NT)
-        for (int sub = 0; sub < TPN; sub++)
-#pragma unroll
-            for (int k = 0; k < 4; k++) snode[i][k] += sacc[(sub * NST + i) * 4 + k];
     __syncthreads();
     // pass C: box ends -> the first state attaining each (ties: lowest stencil index)
     if (tid == 0) {
         for (int c = 0; c < 4; c++) {
-            const int d = c >> 1, up = c & 1;
-            int best = 0;
-            double b = up ? sP[0].U[d] + ph.k * sP[0].sq : sP[0].U[d] - ph.k * sP[0].sq;
-            for (int i = 1; i < NST; i++) {
-                const double v = up ? sP[i].U[d] + ph.k * sP[i].sq : sP[i].U[d] - ph.k * sP[i].sq;
-                if (up ? v > b : v < b) { b = v; best = i; }
-            }
+            const int d = c >> 1, up = c & 1, best = sbest[c];
             const double cb = sbb[c];
             snode[best][1 + d] += cb;
             snode[best][3] += (up ? 0.5 : -0.5) * ph.k * cb / sP[best].sq;
@@ -437,6 +489,8 @@ struct StageVjpSmem {
     double sxb[EPB_L][NV];   // cotangent of the extreme point of Eq. 37 of each component
     int staken[EPB_L], sapm[EPB_L], svstar[EPB_L], sxpt[EPB_L][NV];
     double sW[NS];
+    double sPp[EPB_L][NS + NFP];                        // pressures of w~ over V
+    double spart[EPB_L][NV][4][2];                      // partial sums of step 7
 };
 
 template <int N>
@@ -522,26 +576,33 @@ k_stage_vjp(int stage, double dt, const double* __restrict__ wn, const double* _
         sm.sxarg[ell][v][1] = amn;
     }
     __syncthreads();
-    // 4. alpha (Eq. 39; the lowest component wins ties), P_min over V of w~ (Eq. 47; the
+    // 4. alpha (Eq. 39; the lowest component wins ties), the pressures of w~ over V, a thread per
+    //    point (one thread per element took 32 in turn, most of the kernel's time), P_min (Eq. 47; the
     //    first point wins ties) and the re-limit decision of Eq. 48-49
-    if (tid < EPB_L && e0 + tid < E) {
-        const int ell = tid;
-        double a = 1.0;
+    for (int t = tid; t < EPB_L * NVP; t += NT) {
+        const int ell = t / NVP, n2 = t % NVP;
+        if (e0 + ell >= E) continue;
+        double a = 1.0, q[NV];
         int vs = -1;
         for (int v = 0; v < NV; v++)
             if (sm.salpha_v[ell][v] < a) { a = sm.salpha_v[ell][v]; vs = v; }
-        sm.salpha[ell] = a;
-        sm.svstar[ell] = vs;
+        if (n2 == 0) {
+            sm.salpha[ell] = a;
+            sm.svstar[ell] = vs;
+        }
+        for (int v = 0; v < NV; v++) {
+            const double mv = smean[ell][v], av = ph.uncoupled ? sm.salpha_v[ell][v] : a;
+            q[v] = mv + av * ((n2 < NS ? sw[ell][v][n2] : sf[ell][v][n2 - NS]) - mv);
+        }
+        sm.sPp[ell][n2] = kbl_pressure<2>(q, gm1);
+    }
+    __syncthreads();
+    if (tid < EPB_L && e0 + tid < E) {
+        const int ell = tid;
         double pmin = INFINITY, q[NV];
         int apm = 0;
-        for (int n2 = 0; n2 < NVP; n2++) {
-            for (int v = 0; v < NV; v++) {
-                const double mv = smean[ell][v], av = ph.uncoupled ? sm.salpha_v[ell][v] : a;
-                q[v] = mv + av * ((n2 < NS ? sw[ell][v][n2] : sf[ell][v][n2 - NS]) - mv);
-            }
-            const double P = kbl_pressure<2>(q, gm1);
-            if (P < pmin) { pmin = P; apm = n2; }
-        }
+        for (int n2 = 0; n2 < NVP; n2++)
+            if (sm.sPp[ell][n2] < pmin) { pmin = sm.sPp[ell][n2]; apm = n2; }
         int taken = 0;
         double aP = 1.0, Pbar = 0.0;
         if (pmin < ph.p_floor) {
@@ -604,23 +665,29 @@ k_stage_vjp(int stage, double dt, const double* __restrict__ wn, const double* _
     }
     __syncthreads();
     // 7. Eq. 38 backwards: the cotangent of each component's factor (summed into alpha_min's
-    //    when coupled), then Eq. 37 through the winning ratio
+    //    when coupled; four threads share a component's points), then Eq. 37 through the winning ratio
+    for (int t = tid; t < EPB_L * NV * 4; t += NT) {
+        const int ell = t / (NV * 4), v = (t / 4) % NV, part = t % 4;
+        if (e0 + ell >= E) continue;
+        const double mv = smean[ell][v];
+        double st = 0.0, ab = 0.0;
+        for (int n2 = part; n2 < NVP; n2 += 4) {
+            const double c = n2 < NS ? stb[ell][v][n2] : stfb[ell][v][n2 - NS];
+            st += c;
+            ab += c * ((n2 < NS ? sw[ell][v][n2] : sf[ell][v][n2 - NS]) - mv);
+        }
+        sm.spart[ell][v][part][0] = st;
+        sm.spart[ell][v][part][1] = ab;
+    }
+    __syncthreads();
     if (tid < EPB_L && e0 + tid < E) {
         const int ell = tid, ee = e0 + ell;
         double abv[NV];
         for (int v = 0; v < NV; v++) {
-            const double mv = smean[ell][v], av = aeff(ell, v);
-            double st = 0.0, ab = 0.0;
-            for (int n2 = 0; n2 < NS; n2++) {
-                st += stb[ell][v][n2];
-                ab += stb[ell][v][n2] * (sw[ell][v][n2] - mv);
-            }
-            for (int fp = 0; fp < NFP; fp++) {
-                st += stfb[ell][v][fp];
-                ab += stfb[ell][v][fp] * (sf[ell][v][fp] - mv);
-            }
-            smb[ell][v] += (1.0 - av) * st;
-            abv[v] = ab;
+            const double av = aeff(ell, v);
+            const auto& p = sm.spart[ell][v];
+            smb[ell][v] += (1.0 - av) * ((p[0][0] + p[1][0]) + (p[2][0] + p[3][0]));
+            abv[v] = (p[0][1] + p[1][1]) + (p[2][1] + p[3][1]);
             sm.sxpt[ell][v] = -1;
             sm.sxb[ell][v] = 0.0;
         }
