@@ -227,13 +227,14 @@ cudaError_t dalloc(T** p, size_t count)
 // then per stage the residual, the bounds and the stage + limiter kernel, which also writes the
 // next stage's traces (stages 0 and 1) or advances the clock (stage 2).  Without a side stream:
 // 10 ordinary launches in one chain (traces and time step in one kernel).  With a side stream s2
-// and its events (ctx->pdl set): the time step runs on the side branch beside the traces, and the
-// main chain's kernels (traces, residual, bounds, stage) are programmatic dependents, each
-// waiting for its predecessor before it touches memory and letting its own dependent launch at
-// once; the stage kernel waits only before it reads the bounds (kbl_limit_body.cuh), so its
-// combination and screen overlap the bounds launch's last blocks: 11 kernels.  A residual on a
-// branch beside the bounds measured no better than in the chain: the bounds kernel holds the
-// issue slots and the residency either way.
+// and its events (ctx->pdl set), 11 kernels on two branches: the time step beside the traces, then
+// each stage's residual beside its bounds (both read only the state and its traces); the stage
+// kernel joins them.  Traces and bounds are programmatic dependents on the main branch: a bounds
+// block is resident when the stage before it ends.  The stage kernel is an ordinary launch behind
+// both.  Step time against one main chain traces -> residual -> bounds -> stage of programmatic
+// dependents: 200 1D P3 elements in FP64 82 us there, 62 here; 16^2 P3 mixed 51 and 45, 32^2 FP64
+// 274 and 243; at 128^2 the bounds fill the chip and little is left to hide: mixed 515 and 513,
+// FP64 3025 and 3001 (so no rule on the size).
 int issue_step(kbl_ctx* c, double* w, double cfl, cudaStream_t s, cudaStream_t s2 = nullptr,
                cudaEvent_t* ev = nullptr)
 {
@@ -241,7 +242,7 @@ int issue_step(kbl_ctx* c, double* w, double cfl, cudaStream_t s, cudaStream_t s
     if (s2) {
         // the time step on the side branch, beside the traces: only the stage kernels read it, and
         // they run after the branch joins (the first residual follows it on the same stream)
-        if (cudaEventRecord(ev[6], s) != cudaSuccess || cudaStreamWaitEvent(s2, ev[6], 0) != cudaSuccess) return -1;
+        if (cudaEventRecord(ev[2], s) != cudaSuccess || cudaStreamWaitEvent(s2, ev[2], 0) != cudaSuccess) return -1;
         if ((r = launch_dt_step(c, w, cfl, s2)) < 0) return -1;
         n += r;
         if ((r = launch_traces(c, w, c->d_wf, s)) < 0) return -1;
@@ -253,16 +254,18 @@ int issue_step(kbl_ctx* c, double* w, double cfl, cudaStream_t s, cudaStream_t s
     const double* wn = w;
     const double* ws = w;
     double* outs[3] = {c->d_wa, c->d_wb, w};
-    // with a side stream the main chain is residual -> bounds -> stage per stage, each a
-    // programmatic dependent of the one before; the time step (side branch) joins before the
-    // first residual
-    if (s2 && cudaEventRecord(ev[0], s2) != cudaSuccess) return -1;
     for (int st = 0; st < 3; st++) {
-        if (s2 && st == 0 && cudaStreamWaitEvent(s, ev[0], 0) != cudaSuccess) return -1;
-        if ((r = launch_rhs(c, ws, c->d_wf, c->d_R, s)) < 0) return -1;
+        if (s2) {   // the residual on the side branch, behind the traces (stage 0: and the time step)
+            if (cudaEventRecord(ev[0], s) != cudaSuccess || cudaStreamWaitEvent(s2, ev[0], 0) != cudaSuccess) return -1;
+            if ((r = launch_rhs(c, ws, c->d_wf, c->d_R, s2)) < 0) return -1;
+            if (cudaEventRecord(ev[1], s2) != cudaSuccess) return -1;
+        } else if ((r = launch_rhs(c, ws, c->d_wf, c->d_R, s)) < 0) {
+            return -1;
+        }
         n += r;
         if ((r = launch_bounds(c, ws, c->d_wf, c->d_bnd, s)) < 0) return -1;
         n += r;
+        if (s2 && cudaStreamWaitEvent(s, ev[1], 0) != cudaSuccess) return -1;
         if ((r = launch_stage_step(c, st, wn, ws, c->d_R, c->d_bnd, outs[st], st < 2 ? c->d_wf : nullptr, st == 2, s)) <
             0)
             return -1;
@@ -637,18 +640,18 @@ kbl_status kbl_step(kbl_ctx* c, double* w, double cfl)
         c->graph = nullptr;
         c->graph_w = nullptr;
         cudaStream_t cap = nullptr, side = nullptr;
-        cudaEvent_t ev[7] = {};
+        cudaEvent_t ev[3] = {};
         cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
-        // the side branch (the time step, beside the first traces) at the highest priority, so
+        // the side branch (time step and residuals) at the highest priority, so
         // that its blocks are placed before the traces kernel's later blocks
         int prio_lo = 0, prio_hi = 0;
         if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
         if (e == cudaSuccess && c->overlap_rhs)
             e = cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, prio_hi);
-        for (int k = 0; k < 7 && e == cudaSuccess && side; k++)
+        for (int k = 0; k < 3 && e == cudaSuccess && side; k++)
             e = cudaEventCreateWithFlags(&ev[k], cudaEventDisableTiming);
         auto release = [&]() {
-            for (int k = 0; k < 7; k++)
+            for (int k = 0; k < 3; k++)
                 if (ev[k]) cudaEventDestroy(ev[k]);
             if (side) cudaStreamDestroy(side);
             if (cap) cudaStreamDestroy(cap);
@@ -662,7 +665,7 @@ kbl_status kbl_step(kbl_ctx* c, double* w, double cfl)
             release();
             return cuda_fail(c, e, "begin capture");
         }
-        c->pdl = side != nullptr;   // the main chain of the branched graph as programmatic dependents
+        c->pdl = side != nullptr;   // traces and bounds of the branched graph as programmatic dependents
         const int n = issue_step(c, w, cfl, cap, side, ev);
         c->pdl = false;
         cudaGraph_t g = nullptr;

@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(B2f64<NX>::NT, B2f64<NX>::MINB)
 k_bounds2d_f64(const double* __restrict__ w, const double* __restrict__ wf, MeshDev m, Phys ph,
                double* __restrict__ bnd, DevFlags* flags)
 {
+    kbl_grid_dep_sync();
     constexpr int NST = N * N + 8 * N, NT = B2f64<NX>::NT;
     const int e = blockIdx.x;
     bounds2d_f64_core<NST, NX>(kbl_dyn_smem<Bounds2dF64Smem<NST, NX>>(),
@@ -64,6 +65,7 @@ __global__ void __launch_bounds__(B2pair<NX>::NT, B2pair<NX>::MINB)
 k_bounds2d_pair(const double* __restrict__ w, const double* __restrict__ wf, MeshDev m, Phys ph,
                 double* __restrict__ bnd, DevFlags* flags)
 {
+    kbl_grid_dep_sync();
     constexpr int NST = N * N + 8 * N, NT = B2pair<NX>::NT;
     const int e = blockIdx.x;
     bounds2d_pair_core<NST, NX>(kbl_dyn_smem<Bounds2dPairSmem<NST, NX>>(),
@@ -94,6 +96,7 @@ __global__ void __launch_bounds__(NT)
 k_bounds1d_f64(const double* __restrict__ w, const double* __restrict__ wf, MeshDev m, Phys ph,
                double* __restrict__ bnd, DevFlags* flags)
 {
+    kbl_grid_dep_sync();
     constexpr int NST = WIDE ? 3 * N : N + 4;
     __shared__ Bounds1dSmem<NST, NT> sm;
     const int e = blockIdx.x;
@@ -123,6 +126,7 @@ __global__ void __launch_bounds__(NT1)
 k_bounds1d_f32(const double* __restrict__ w, const double* __restrict__ wf, MeshDev m, Phys ph,
                double* __restrict__ bnd, DevFlags* flags)
 {
+    kbl_grid_dep_sync();
     constexpr int NS = N, NFP = 2, NST = WIDE ? 3 * NS : NS + 2 * NFP, NV = 3;
     constexpr int NW = NT1 / 32;
     __shared__ double sS[NST][NV];
@@ -224,7 +228,7 @@ int run2d(const kbl_ctx* c, const double* w, const double* wf, double* bnd, cuda
 template <int N, int NX>
 int run2d_f64(const kbl_ctx* c, const double* w, const double* wf, double* bnd, cudaStream_t s)
 {
-    kbl_launch_dyn<Bounds2dF64Smem<N * N + 8 * N, NX>>(k_bounds2d_f64<N, NX>, c->E, B2f64<NX>::NT, s, w, wf, mesh_of(c),
+    kbl_launch_dyn<Bounds2dF64Smem<N * N + 8 * N, NX>>(k_bounds2d_f64<N, NX>, c->E, B2f64<NX>::NT, s, c->pdl, w, wf, mesh_of(c),
                                                        c->phys, bnd, c->d_flags);
     return 1;
 }
@@ -232,7 +236,7 @@ int run2d_f64(const kbl_ctx* c, const double* w, const double* wf, double* bnd, 
 template <int N, int NX>
 int run2d_pair(const kbl_ctx* c, const double* w, const double* wf, double* bnd, cudaStream_t s)
 {
-    kbl_launch_dyn<Bounds2dPairSmem<N * N + 8 * N, NX>>(k_bounds2d_pair<N, NX>, c->E, B2pair<NX>::NT, s, w, wf,
+    kbl_launch_dyn<Bounds2dPairSmem<N * N + 8 * N, NX>>(k_bounds2d_pair<N, NX>, c->E, B2pair<NX>::NT, s, c->pdl, w, wf,
                                                         mesh_of(c), c->phys, bnd, c->d_flags);
     return 1;
 }
@@ -245,14 +249,14 @@ int run_bounds(const kbl_ctx* c, const double* w, const double* wf, double* bnd,
         const bool wide = c->cfg.stencil == 1;
         const MeshDev m = mesh_of(c);
         if (c->cfg.precision == KBL_FP32_MIXED) {
-            if (wide) k_bounds1d_f32<N, true><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
-            else k_bounds1d_f32<N><<<c->E, NT1, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+            if (wide) kbl_launch(k_bounds1d_f32<N, true>, c->E, NT1, 0, s, c->pdl, w, wf, m, c->phys, bnd, c->d_flags);
+            else kbl_launch(k_bounds1d_f32<N>, c->E, NT1, 0, s, c->pdl, w, wf, m, c->phys, bnd, c->d_flags);
         } else if (c->cfg.nu[0] <= 64) {   // a thread per node where that many suffice
-            if (wide) k_bounds1d_f64<N, 64, true><<<c->E, 64, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
-            else k_bounds1d_f64<N, 64><<<c->E, 64, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+            if (wide) kbl_launch(k_bounds1d_f64<N, 64, true>, c->E, 64, 0, s, c->pdl, w, wf, m, c->phys, bnd, c->d_flags);
+            else kbl_launch(k_bounds1d_f64<N, 64>, c->E, 64, 0, s, c->pdl, w, wf, m, c->phys, bnd, c->d_flags);
         } else {
-            if (wide) k_bounds1d_f64<N, 256, true><<<c->E, 256, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
-            else k_bounds1d_f64<N, 256><<<c->E, 256, 0, s>>>(w, wf, m, c->phys, bnd, c->d_flags);
+            if (wide) kbl_launch(k_bounds1d_f64<N, 256, true>, c->E, 256, 0, s, c->pdl, w, wf, m, c->phys, bnd, c->d_flags);
+            else kbl_launch(k_bounds1d_f64<N, 256>, c->E, 256, 0, s, c->pdl, w, wf, m, c->phys, bnd, c->d_flags);
         }
         return 1;
     }

@@ -1304,13 +1304,14 @@ __device__ __forceinline__ SM& kbl_dyn_smem()
     return *reinterpret_cast<SM*>(kbl_smem_bytes);
 }
 
-// Launch one block per element with a shared-memory object SM (above 48 KB by opt-in).
+// Launch one block per element with a shared-memory object SM (above 48 KB by opt-in); with pdl, as a
+// programmatic dependent (kbl_launch).
 template <typename SM, typename... KArgs, typename... Args>
-void kbl_launch_dyn(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args)
+void kbl_launch_dyn(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, bool pdl, Args... args)
 {
     if (sizeof(SM) > 48 * 1024)
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM));
-    kernel<<<grid, block, sizeof(SM), s>>>(args...);
+    kbl_launch(kernel, grid, block, sizeof(SM), s, pdl, args...);
 }
 
 }  // namespace kbl_dev

@@ -86,7 +86,7 @@ inline void kbl_phys_derive(Phys& p)
     p.rel_hif = (float)p.rel_hi;
 }
 
-// Programmatic dependent launch inside a step graph: a kernel of the step's main chain first
+// Programmatic dependent launch inside a step graph: a bounds kernel of the step's main branch first
 // waits until the grids it depends on have completed and their writes are visible (it reads
 // their outputs and overwrites buffers they read), then lets its own dependent grid be
 // launched, whose blocks take SM slots as this grid's blocks retire and wait there in turn.
@@ -286,9 +286,9 @@ struct kbl_ctx {
     double* d_qw = nullptr;     // velocity quadrature weights (Romberg), or nullptr
     float* d_tcop = nullptr;    // split residual operator of the tensor-core residual, or nullptr
     int rhs_tc = 0;             // knob: 1 residual products on the tensor cores where covered, 0 CUDA cores
-    int overlap_rhs = 1;        // knob: 1 each stage's residual on a graph branch beside its bounds
-    mutable bool pdl = false;   // set while the branched step graph is captured: the main chain's
-                                // launches are programmatic dependents (kbl_grid_dep_sync)
+    int overlap_rhs = 1;        // knob: 1 the step graph has a side branch (time step, residuals)
+    mutable bool pdl = false;   // set while the branched step graph is captured: its traces and
+                                // bounds are programmatic dependents (kbl_grid_dep_sync)
     std::string err;
     int64_t launches = 0;
     int bounds_tile = 0;        // FP32 bounds thread tile: 0 = 4x4 nodes, 1 = 4x2 nodes

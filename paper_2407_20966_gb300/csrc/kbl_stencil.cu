@@ -74,7 +74,7 @@ int run_stencil(const kbl_ctx* c, int E, int nst, const double* S, double* bnd, 
 template <int NSTC, int NX>
 int run_stencil_f64(const kbl_ctx* c, int E, int nst, const double* S, double* bnd, cudaStream_t s)
 {
-    kbl_launch_dyn<Bounds2dF64Smem<NSTC, NX>>(k_bounds_stencil_f64<NSTC, NX>, E, B2f64<NX>::NT, s, S, nst, E, c->phys, bnd,
+    kbl_launch_dyn<Bounds2dF64Smem<NSTC, NX>>(k_bounds_stencil_f64<NSTC, NX>, E, B2f64<NX>::NT, s, false, S, nst, E, c->phys, bnd,
                                               c->d_flags);
     return 1;
 }
@@ -82,7 +82,7 @@ int run_stencil_f64(const kbl_ctx* c, int E, int nst, const double* S, double* b
 template <int NSTC, int NX>
 int run_stencil_pair(const kbl_ctx* c, int E, int nst, const double* S, double* bnd, cudaStream_t s)
 {
-    kbl_launch_dyn<Bounds2dPairSmem<NSTC, NX>>(k_bounds_stencil_pair<NSTC, NX>, E, B2pair<NX>::NT, s, S, nst, E, c->phys,
+    kbl_launch_dyn<Bounds2dPairSmem<NSTC, NX>>(k_bounds_stencil_pair<NSTC, NX>, E, B2pair<NX>::NT, s, false, S, nst, E, c->phys,
                                                bnd, c->d_flags);
     return 1;
 }

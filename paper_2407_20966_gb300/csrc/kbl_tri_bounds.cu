@@ -90,7 +90,7 @@ void run_tri(const kbl_ctx* c, int E, const TriGather& a, double* bnd, cudaStrea
 template <int NSTC, int NX>
 int run_tri_f64(const kbl_ctx* c, int E, const TriGather& a, double* bnd, cudaStream_t s)
 {
-    kbl_launch_dyn<Bounds2dF64Smem<NSTC, NX>>(k_bounds_tri_f64<NSTC, NX>, E, B2f64<NX>::NT, s, a, E, c->phys, bnd,
+    kbl_launch_dyn<Bounds2dF64Smem<NSTC, NX>>(k_bounds_tri_f64<NSTC, NX>, E, B2f64<NX>::NT, s, false, a, E, c->phys, bnd,
                                               c->d_flags);
     return 1;
 }
@@ -98,7 +98,7 @@ int run_tri_f64(const kbl_ctx* c, int E, const TriGather& a, double* bnd, cudaSt
 template <int NSTC, int NX>
 int run_tri_pair(const kbl_ctx* c, int E, const TriGather& a, double* bnd, cudaStream_t s)
 {
-    kbl_launch_dyn<Bounds2dPairSmem<NSTC, NX>>(k_bounds_tri_pair<NSTC, NX>, E, B2pair<NX>::NT, s, a, E, c->phys, bnd,
+    kbl_launch_dyn<Bounds2dPairSmem<NSTC, NX>>(k_bounds_tri_pair<NSTC, NX>, E, B2pair<NX>::NT, s, false, a, E, c->phys, bnd,
                                                c->d_flags);
     return 1;
 }
