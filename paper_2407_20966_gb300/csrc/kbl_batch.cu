@@ -233,22 +233,28 @@ template <int N, int NT = NTB>
 __device__ __forceinline__ void stage_item(void* smraw, const ProbDesc& pd, const WorkItem& wi, const FrOps& ops,
                                            const Phys& ph, int stage, const double* wn, const double* ws,
                                            const double* R, const double* bnd, double dt, double* wout,
-                                           DevFlags* flags)
+                                           DevFlags* flags, double* wf_next = nullptr)
 {
     constexpr int EPB = FrEpb<N, NT>::EPB;
     auto& sm = *reinterpret_cast<LimSmem<2, N, EPB>*>(smraw);
     const int e_end = wi.e0 + wi.n;
-    for (int eb = wi.e0; eb < e_end; eb += EPB)
-        stage_limit_block<2, N, EPB>(sm, NT, 0, stage, wn + pd.woff, ws + pd.woff, R + pd.woff,
-                                            bnd + pd.bndoff, dt, wout + pd.woff, nullptr, pd.E, ops, ph, flags, eb,
-                                            min(EPB, e_end - eb));
+    for (int eb = wi.e0; eb < e_end; eb += EPB) {
+        stage_limit_block<2, N, EPB, true>(sm, NT, 0, stage, wn + pd.woff, ws + pd.woff, R + pd.woff, bnd + pd.bndoff,
+                                           dt, wout + pd.woff, nullptr, pd.E, ops, ph, flags, eb, min(EPB, e_end - eb));
+        if (wf_next) traces_of_block<2, N, EPB>(sm, NT, pd.E, eb, min(EPB, e_end - eb), wf_next + pd.wfoff);
+    }
 }
 
+// With wf_next the stage also writes the next stage's face traces from the limited state in shared
+// memory.  Launches of their own for stages 1 and 2 read the state back, 165 us each for 96 problems
+// of 16^2 to 64^2 elements; here their FP64 work overlaps the stage's memory traffic: step 6.34 ->
+// 6.16 ms.
 // 4 resident blocks: without the hint the switch over orders inflates the register count
 __global__ void __launch_bounds__(NTB, 4) k_batch_stage(BatchDev bd, const WorkItem* __restrict__ items, int n_items,
                                                      unsigned* counter, BatchOps ops, Phys ph, int stage,
                                                      const double* wn, const double* ws, const double* R,
-                                                     const double* bnd, const double* dt, double* wout, DevFlags* flags)
+                                                     const double* bnd, const double* dt, double* wout, DevFlags* flags,
+                                                     double* wf_next)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int s_item;
@@ -259,10 +265,10 @@ __global__ void __launch_bounds__(NTB, 4) k_batch_stage(BatchDev bd, const WorkI
         const ProbDesc pd = bd.probs[wi.prob];
         const double dtp = dt[wi.prob];
         switch (pd.p) {
-            case 1: stage_item<2>(smraw, pd, wi, ops.o[1], ph, stage, wn, ws, R, bnd, dtp, wout, flags); break;
-            case 2: stage_item<3>(smraw, pd, wi, ops.o[2], ph, stage, wn, ws, R, bnd, dtp, wout, flags); break;
-            case 3: stage_item<4>(smraw, pd, wi, ops.o[3], ph, stage, wn, ws, R, bnd, dtp, wout, flags); break;
-            case 4: stage_item<5>(smraw, pd, wi, ops.o[4], ph, stage, wn, ws, R, bnd, dtp, wout, flags); break;
+            case 1: stage_item<2>(smraw, pd, wi, ops.o[1], ph, stage, wn, ws, R, bnd, dtp, wout, flags, wf_next); break;
+            case 2: stage_item<3>(smraw, pd, wi, ops.o[2], ph, stage, wn, ws, R, bnd, dtp, wout, flags, wf_next); break;
+            case 3: stage_item<4>(smraw, pd, wi, ops.o[3], ph, stage, wn, ws, R, bnd, dtp, wout, flags, wf_next); break;
+            case 4: stage_item<5>(smraw, pd, wi, ops.o[4], ph, stage, wn, ws, R, bnd, dtp, wout, flags, wf_next); break;
         }
     }
 }
@@ -703,7 +709,10 @@ int issue_batch_step(kbl_batch* b, double* w, double cfl, cudaStream_t s, const 
     const double* ws = w;
     double* outs[3] = {b->d_wa, b->d_wb, w};
     for (int st = 0; st < 3; st++) {
-        k_batch_traces<<<g_tr, NTB, 0, s>>>(bd, is.fr, is.n_fr, is.counters + 1 + 4 * st, b->ops, ws, b->d_wf);
+        if (st == 0) {   // the later stages' traces are written by the stage kernel before them
+            k_batch_traces<<<g_tr, NTB, 0, s>>>(bd, is.fr, is.n_fr, is.counters + 1, b->ops, ws, b->d_wf);
+            n++;
+        }
         cudaStream_t sr = s;
         if (s2) {
             cudaEventRecord(ev[2 * st], s);
@@ -717,8 +726,8 @@ int issue_batch_step(kbl_batch* b, double* w, double cfl, cudaStream_t s, const 
         if (s2) cudaStreamWaitEvent(s, ev[2 * st + 1], 0);
         k_batch_stage<<<g_st, NTB, sizeof(LimUnion<>), s>>>(bd, is.fr, is.n_fr, is.counters + 4 + 4 * st, b->ops,
                                                           b->phys, st, wn, ws, b->d_R, b->d_bnd, b->d_dt, outs[st],
-                                                          b->d_flags);
-        n += 3;
+                                                          b->d_flags, st < 2 ? b->d_wf : nullptr);
+        n += 2;
         ws = outs[st];
     }
     k_batch_time_advance<<<(np + 255) / 256, 256, 0, s>>>(b->d_dt + is.p0, b->d_t + is.p0, np);
@@ -1203,7 +1212,7 @@ kbl_status kbl_batch_stage(kbl_batch* b, int st, const double* wn, const double*
     cudaMemsetAsync(b->d_counters, 0, NCOUNTERS * sizeof(unsigned), s);
     k_batch_stage<<<grid_of(b, fr_blocks_per_sm((const void*)k_batch_stage, sizeof(LimUnion<>))), NTB, sizeof(LimUnion<>),
                     s>>>(dev_of(b), b->d_fr_items, b->n_fr_items, b->d_counters + 4, b->ops, b->phys, st, wn, ws, R,
-                         bnd, dt_dev, wout, b->d_flags);
+                         bnd, dt_dev, wout, b->d_flags, nullptr);
     b->launches += 1;
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? KBL_OK : bfail(b, KBL_ECUDA, cudaGetErrorString(e));
