@@ -29,7 +29,7 @@ using namespace kbl_dev;
 constexpr int PMAX_B = 4;        // orders 1..4
 constexpr int NX_B = 32;         // velocity points per axis supported by the batch
 constexpr int NTB = 256;         // threads per block of the FR / limiter phases
-constexpr int FR_CHUNK = 256;    // elements per work item of the FR / limiter phases
+constexpr int RESIDENT_FR = 4;   // resident blocks per SM of the FR / limiter phases
 constexpr int NCOUNTERS = 16;    // one work counter per persistent launch of a step
 #define KBL_BATCH_HOST_GROUPS 8  // problem groups of kbl_batch_run_host (copies overlap steps)
 
@@ -549,6 +549,7 @@ struct kbl_batch {
     unsigned* d_counters = nullptr;
     WorkItem* d_fr_items = nullptr;
     int n_fr_items = 0;
+    int fr_passes = 1;                   // block passes (fr_epb elements each) per FR work item
     WorkItem* d_b_items = nullptr;       // bounds items for the current chunk size
     int n_b_items = 0;
     // launch shape of the bounds phase
@@ -606,12 +607,16 @@ size_t bounds_smem(int tile)
     return tile == 2 ? sizeof(BoundsUnion<3>) : tile == 1 ? sizeof(BoundsUnion<2>) : sizeof(BoundsUnion<0>);
 }
 
-std::vector<WorkItem> make_items(const std::vector<ProbDesc>& probs, int chunk, int p0 = 0, int p1 = -1)
+// Work items of problems [p0, p1): chunk_of(p) elements of one problem of order p each.
+template <typename ChunkOf>
+std::vector<WorkItem> make_items_by(const std::vector<ProbDesc>& probs, ChunkOf chunk_of, int p0 = 0, int p1 = -1)
 {
     std::vector<WorkItem> items;
     if (p1 < 0) p1 = (int)probs.size();
-    for (int pi = p0; pi < p1; pi++)
+    for (int pi = p0; pi < p1; pi++) {
+        const int chunk = chunk_of(probs[pi].p);
         for (int e0 = 0; e0 < probs[pi].E; e0 += chunk) items.push_back({pi, e0, std::min(chunk, probs[pi].E - e0)});
+    }
     // expensive first: higher order, then fuller items
     std::stable_sort(items.begin(), items.end(), [&](const WorkItem& a, const WorkItem& b) {
         const int pa = probs[a.prob].p, pb = probs[b.prob].p;
@@ -619,6 +624,32 @@ std::vector<WorkItem> make_items(const std::vector<ProbDesc>& probs, int chunk, 
         return a.n > b.n;
     });
     return items;
+}
+
+std::vector<WorkItem> make_items(const std::vector<ProbDesc>& probs, int chunk, int p0 = 0, int p1 = -1)
+{
+    return make_items_by(probs, [=](int) { return chunk; }, p0, p1);
+}
+
+// Elements that a block of the FR / limiter phases works on at a time (FrEpb).
+int fr_epb(int p) { return NTB / ((p + 1) * (p + 1)); }
+
+std::vector<WorkItem> make_fr_items(const std::vector<ProbDesc>& probs, int fr_passes, int p0 = 0, int p1 = -1)
+{
+    return make_items_by(probs, [=](int p) { return fr_passes * fr_epb(p); }, p0, p1);
+}
+
+// Block passes per FR work item: as many as leave every resident block about six items, eight at
+// most.  An item of fixed size (256 elements, 4 to 26 passes by order) left a batch of 96 problems of
+// 16^2 to 64^2 elements one item per block and its last P4 items running alone; one pass alone costs
+// small batches least and large ones an item's two barriers and loads per pass.  Step of that batch,
+// 1 / 2 / 4 / 8 / 16 passes: 5.75 / 5.72 / 5.81 / 6.04 / 6.44 ms (6.28 with 256 elements); of 12
+// problems of 12^2 to 40^2: 0.80 / 0.86 / 0.91 / 1.04 / 1.26 (bounds items of 16 elements).
+int fr_passes_for(const kbl_batch* b)
+{
+    long long passes = 0;
+    for (const auto& pr : b->probs) passes += (pr.E + fr_epb(pr.p) - 1) / fr_epb(pr.p);
+    return (int)std::min(8LL, std::max(1LL, passes / (6LL * RESIDENT_FR * b->nsm)));
 }
 
 cudaError_t upload_items(kbl_batch* b, const std::vector<WorkItem>& items, WorkItem** d, int* n)
@@ -787,7 +818,8 @@ cudaError_t upload_counts(kbl_batch* b)
 {
     std::vector<int> cnt(2 * (size_t)b->P, 0);
     for (int i = 0; i < b->P; i++) {
-        cnt[i] = (b->probs[i].E + FR_CHUNK - 1) / FR_CHUNK;
+        const int fc = b->fr_passes * fr_epb(b->probs[i].p);
+        cnt[i] = (b->probs[i].E + fc - 1) / fc;
         cnt[b->P + i] = (b->probs[i].E + b->chunk - 1) / b->chunk;
     }
     cudaError_t e = cudaSuccess;
@@ -846,6 +878,16 @@ void drop_graph(kbl_batch* b)
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
     b->graph_w = nullptr;
+}
+
+// Bounds phase before the autotuner: the 4 x 2 thread tile, and as many elements per item as leave
+// every resident block about sixteen items, 16 at most.  Step with 1 / 4 / 8 / 16 elements: 2 problems
+// of 8^2 to 12^2 elements 103 / 178 / 267 / 431 us, 12 of 12^2 to 40^2 329 / 350 / 473 / 807, 96 of
+// 16^2 to 64^2 5876 / 5719 / 5714 / 5751.
+constexpr int BOUNDS_TILE = 1;
+int bounds_chunk_for(const kbl_batch* b, int per_sm)
+{
+    return (int)std::min(16LL, std::max(1LL, b->E_total / (16LL * per_sm * b->nsm)));
 }
 
 cudaError_t set_bounds_shape(kbl_batch* b, int tile, int chunk, int per_sm)
@@ -987,10 +1029,12 @@ kbl_status kbl_batch_create(kbl_batch** out, const kbl_config* cfg, int P, const
     if (e == cudaSuccess && bcoff > 0) e = cudaMemcpy(b->d_bc, bc, bcoff * 4 * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->d_flags, 0, sizeof(DevFlags));
     if (e == cudaSuccess) e = cudaMemset(b->d_t, 0, P * sizeof(double));
-    if (e == cudaSuccess) e = upload_items(b, make_items(b->probs, FR_CHUNK), &b->d_fr_items, &b->n_fr_items);
+    b->fr_passes = fr_passes_for(b);
+    if (e == cudaSuccess) e = upload_items(b, make_fr_items(b->probs, b->fr_passes), &b->d_fr_items, &b->n_fr_items);
     if (e == cudaSuccess) {
         cudaFuncSetAttribute(k_batch_stage, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LimUnion<>));
-        e = set_bounds_shape(b, 1, 16, max_bounds_blocks(1));
+        const int per_sm = max_bounds_blocks(BOUNDS_TILE);
+        e = set_bounds_shape(b, BOUNDS_TILE, bounds_chunk_for(b, per_sm), per_sm);
     }
     if (e != cudaSuccess) {
         kbl_batch_destroy(b);
@@ -1082,7 +1126,7 @@ cudaError_t build_groups(kbl_batch* b)
         gr.p0 = p0;
         gr.p1 = p1;
         gr.chunk = b->chunk;
-        cudaError_t e = upload_items(b, make_items(b->probs, FR_CHUNK, p0, p1), &gr.fr, &gr.n_fr);
+        cudaError_t e = upload_items(b, make_fr_items(b->probs, b->fr_passes, p0, p1), &gr.fr, &gr.n_fr);
         if (e == cudaSuccess) e = upload_items(b, make_items(b->probs, b->chunk, p0, p1), &gr.bi, &gr.n_bi);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&gr.h2d, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&gr.done, cudaEventDisableTiming);

@@ -296,3 +296,40 @@ def test_batch_one_launch_wait_timeout_is_reported():
     b.step(wd, 0.1)
     b.check()
     np.testing.assert_array_equal(wd.cpu().numpy(), wref.cpu().numpy())
+
+
+@pytest.mark.parametrize("p,nx,ny", [(1, 1, 1), (1, 9, 7), (1, 8, 8), (1, 13, 5), (2, 7, 4), (2, 29, 1), (3, 4, 4),
+                                     (3, 17, 1), (4, 5, 2), (4, 11, 1), (4, 320, 310)])
+def test_batch_work_items_at_their_edges(p, nx, ny):
+    """Element counts at, below and above one block's share (64, 28, 16 and 10 elements of P1 to P4)
+    beside one small problem, and a batch of enough elements for several passes per work item
+    (99,200 P4 elements): both forms of the step equal the single-mesh step bit for bit."""
+    import torch
+    from paper_2407_20966_gb300 import kbl
+
+    def waves(x, y):   # within 0.2 of a uniform state, so that its traces are physical on any mesh
+        rho = 1.0 + 0.1 * np.sin(2 * np.pi * x) * np.cos(2 * np.pi * y)
+        u, v = 0.3 + 0.1 * np.cos(2 * np.pi * y), -0.2 + 0.1 * np.sin(2 * np.pi * x)
+        return np.stack([rho, rho * u, rho * v, 2.5 + 0.5 * rho * (u * u + v * v)])
+    meshes = [inputs.mesh_2d(nx, ny, 0.0, 1.0, 0.0, 1.0, periodic=(True, True)),
+              inputs.mesh_2d(3, 2, 0.0, 1.0, 0.0, 1.0, periodic=(True, True))]
+    probs = [(p, meshes[0]), (3, meshes[1])]
+    b = kbl.Batch([(q, m.nbr, m.h, m.bc) for q, m in probs])
+    fields = [inputs.nodal_field(m, np.polynomial.legendre.leggauss(q + 1)[0], waves) for q, m in probs]
+    w0 = np.concatenate([f.ravel() for f in fields])
+    for form in (0, 1):
+        b.set_form(form)
+        wd = torch.from_numpy(w0).cuda()
+        b.step(wd, 0.1)
+        b.check()
+        got, dts = wd.cpu().numpy(), b.dt()
+        for i, (q, m) in enumerate(probs):
+            ctx = kbl.Context(dim=2, p=q, nu=(32, 32), precision=kbl.FP32_MIXED)
+            ctx.set_tuning(kbl.TUNE_RHS_TC, 0)
+            ctx.set_tuning(kbl.TUNE_BOUNDS_TILE, b.tuning()["tile"])
+            ctx.mesh_upload(m.nbr, m.h, m.bc)
+            wi = torch.from_numpy(np.ascontiguousarray(fields[i])).cuda()
+            ctx.set_time(0.0)
+            ctx.step(wi, 0.1)
+            assert ctx.time() == dts[i]
+            np.testing.assert_array_equal(b.state_view(got, i), wi.cpu().numpy())
