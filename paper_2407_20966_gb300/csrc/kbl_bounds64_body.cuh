@@ -319,7 +319,8 @@ __device__ __forceinline__ void bounds2d_f64_core(Bounds2dF64Smem<NST, NX>& sm, 
 //   moments      the nodes' values in error-free FP32 sums along rows and columns, those in FP64;
 //                the quadrature weights are in the tables already
 //
-// Measured at 128^2 P3, 32^2 grid: 0.87 ms per launch; 0.95 with the y table's values stored twice (a
+// Measured at 128^2 P3, 32^2 grid: 0.85 ms per launch; 0.87 with both axes' grid coefficients in one
+// thread per state, 0.95 with the y table's values stored twice (a
 // 128-bit shared load takes four wavefronts however many lanes share its addresses, and the passes
 // wait on them: 6.9k of 19k clocks per element), 1.08 with the moments node by node in FP64 and the
 // states' constants in two passes over shared memory, 6.52 for the FP64 kernel above (86% of the FP64
@@ -661,6 +662,58 @@ __device__ __forceinline__ Sum4 sum_lanes(const Sum4x2& a)
     return s;
 }
 
+// Sums of any number of envelope values -M + E over the lanes of a warp, error-free: -m + r + q with m
+// the FP32 sum of the M; r that of the E less the errors of m; q what r lost (2^-48 of the values, so
+// that its own roundings are of no account).  Two sums side by side.
+struct LaneSum2 {
+    float2 m, r, q;
+};
+struct LaneSum {
+    float m, r, q;
+    __device__ __forceinline__ double value() const { return widen_fast(-m) + (widen_fast(r) + widen_fast(q)); }
+};
+__device__ __forceinline__ LaneSum2 lane_pair(float2 Ma, float2 Ea, float2 Mb, float2 Eb)
+{
+    LaneSum2 s;
+    float2 e, r, q1, q2;
+    f2two_sum(Ma, Mb, s.m, e);
+    f2two_sum(Ea, Eb, r, q1);
+    f2two_sum(r, f2neg(e), s.r, q2);
+    s.q = __fadd2_rn(q1, q2);
+    return s;
+}
+__device__ __forceinline__ LaneSum2 lane_merge(const LaneSum2& a, const LaneSum2& b)
+{
+    LaneSum2 s = lane_pair(a.m, a.r, b.m, b.r);
+    s.q = __fadd2_rn(s.q, __fadd2_rn(a.q, b.q));
+    return s;
+}
+// (a.x, b.x) or (a.y, b.y)
+__device__ __forceinline__ LaneSum2 lane_x(const LaneSum2& a, const LaneSum2& b)
+{
+    return {make_float2(a.m.x, b.m.x), make_float2(a.r.x, b.r.x), make_float2(a.q.x, b.q.x)};
+}
+__device__ __forceinline__ LaneSum2 lane_y(const LaneSum2& a, const LaneSum2& b)
+{
+    return {make_float2(a.m.y, b.m.y), make_float2(a.r.y, b.r.y), make_float2(a.q.y, b.q.y)};
+}
+// A step of a reduce-scatter: the lanes with up keep hi and the others lo, each plus its partner's.
+__device__ __forceinline__ LaneSum2 lane_exchange(const LaneSum2& lo, const LaneSum2& hi, bool up, int off)
+{
+    auto swap = [&](float l, float h, float& keep) {
+        keep = up ? h : l;
+        return __shfl_xor_sync(0xffffffffu, up ? l : h, off);
+    };
+    LaneSum2 k, o;
+    o.m.x = swap(lo.m.x, hi.m.x, k.m.x);
+    o.m.y = swap(lo.m.y, hi.m.y, k.m.y);
+    o.r.x = swap(lo.r.x, hi.r.x, k.r.x);
+    o.r.y = swap(lo.r.y, hi.r.y, k.r.y);
+    o.q.x = swap(lo.q.x, hi.q.x, k.q.x);
+    o.q.y = swap(lo.q.y, hi.q.y, k.q.y);
+    return lane_merge(k, o);
+}
+
 // 2^k for |k| <= 1000
 __device__ __forceinline__ double pow2_f64(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
@@ -690,6 +743,7 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
     long long klo[2] = {0x7fffffffffffffffll, 0x7fffffffffffffffll}, khi[2] = {-0x7fffffffffffffffll, -0x7fffffffffffffffll};
     int kA = 0, bad = 0, out_of_range = 0;
     double th = 0.0, rs = 0.0, U[2] = {0.0, 0.0}, A = 0.0;
+    double(*kap)[4] = reinterpret_cast<double(*)[4]>(&sm.u.tab);   // per state kappa and U, until the tables
     if (tid < NST) {
         const double rho = sm.S[tid][0], mx = sm.S[tid][1], my = sm.S[tid][2], En = sm.S[tid][3];
         if (exponent_ok(rho) && exponent_ok(En)) {
@@ -715,9 +769,18 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
             }
             kA = __double2hiint(A);
             out_of_range = !exponent_ok(th);
+            // kappa = sqrt(log2(e) / 2) / sqrt(theta) as kh + kl
+            const double rl = rsqrt_rest(th, rs);
+            const double kh = 0.8493218002880191 * rs;
+            kap[tid][0] = kh;
+            kap[tid][1] =
+                fma(0.8493218002880191, rs, -kh) + fma(-2.5959464104597403e-17, rs, 0.8493218002880191 * rl);
+            kap[tid][2] = U[0];
+            kap[tid][3] = U[1];
         } else {
             bad = !(rho > 0.0) || !(kbl_pressure<2>(sm.S[tid], ph.gamma - 1.0) > 0.0);
             out_of_range = 1;
+            kap[tid][0] = kap[tid][1] = kap[tid][2] = kap[tid][3] = 0.0;
         }
     }
 #pragma unroll
@@ -769,28 +832,30 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
     if (abs(eA) > 900 || abs(eU) > 450) out_of_range = 1;
     const double sA = pow2_f64(abs(eA) > 900 ? 0 : -eA), sU = pow2_f64(abs(eU) > 450 ? 0 : -eU);
 
-    // 2. scaled constants, and the velocity grid's coefficients
+    // 2. scaled constants, and the velocity grid's coefficients: a thread per state and axis where the
+    //    block has as many (FP64 instructions take as long for half a warp as for a whole one, and the
+    //    chain is shorter: 128^2 P3 step 3.01 -> 2.95 ms against a thread per state)
     if (tid < NST) {
         const Triple At = split_f32(A * sA), Ct = split_f32(ph.half_delta2 * th * (sU * sU));
-        // kappa = sqrt(log2(e) / 2) / sqrt(theta) as kh + kl
-        const double rl = rsqrt_rest(th, rs);
-        const double kh = 0.8493218002880191 * rs;
-        const double kl = fma(0.8493218002880191, rs, -kh) + fma(-2.5959464104597403e-17, rs, 0.8493218002880191 * rl);
-        float tm = 0.0f;
-#pragma unroll
-        for (int d = 0; d < 2; d++) {
-            const double hd = sm.h[d], dc = sm.c[d] - U[d];
-            const double zh = dc * kh, dh = hd * kh;
-            // the low parts, below 2^-48, in units of 2^-58 like the high ones
-            const double zl = fma(dc, kl, fma(dc, kh, -zh)), dl = fma(hd, kl, fma(hd, kh, -dh));
-            sm.P[tid].z[d] = fixed58(zh) + fixed58(zl);
-            sm.P[tid].dz[d] = fixed58(dh) + fixed58(dl);
-            // the largest exponent over the box, in FP32 with a margin
-            tm = fmaxf(tm, fabsf(f32_trunc(zh)) + f32_trunc(dh) * (float)(nu / 2 + 1));
-        }
         sm.P[tid].A = At;
         sm.P[tid].C = Ct;
-        if (!(tm < 15.5f) || !(At.h >= 0x1p-60f) || !(Ct.h == 0.0f || (Ct.h >= 0x1p-30f && Ct.h < 0x1p60f))) out_of_range = 1;
+        if (!(At.h >= 0x1p-60f) || !(Ct.h == 0.0f || (Ct.h >= 0x1p-30f && Ct.h < 0x1p60f))) out_of_range = 1;
+    }
+    auto grid_coefficients = [&](int i, int d) {
+        const double kh = kap[i][0], kl = kap[i][1], hd = sm.h[d], dc = sm.c[d] - kap[i][2 + d];
+        const double zh = dc * kh, dh = hd * kh;
+        // the low parts, below 2^-48, in units of 2^-58 like the high ones
+        const double zl = fma(dc, kl, fma(dc, kh, -zh)), dl = fma(hd, kl, fma(hd, kh, -dh));
+        sm.P[i].z[d] = fixed58(zh) + fixed58(zl);
+        sm.P[i].dz[d] = fixed58(dh) + fixed58(dl);
+        // the largest exponent over the box, in FP32 with a margin
+        if (!(fabsf(f32_trunc(zh)) + f32_trunc(dh) * (float)(nu / 2 + 1) < 15.5f)) out_of_range = 1;
+    };
+    if constexpr (2 * NST <= NT) {
+        if (tid < 2 * NST) grid_coefficients(tid < NST ? tid : tid - NST, tid < NST ? 0 : 1);
+    } else if (tid < NST) {
+#pragma unroll
+        for (int d = 0; d < 2; d++) grid_coefficients(tid, d);
     }
     for (int j = NT - 1 - tid; j < 2 * NX; j += NT) {   // from the last thread: the first hold states
         const int d = j / NX, jj = j % NX;
