@@ -1020,59 +1020,117 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
             }
         }
 
-        // 5. moments: the envelopes' two floats meet in error-free FP32 sums (a row over x for the weights
-        //    in v, a column over y for those in u, everything for I), which then enter FP64: a third of
-        //    the FP64 instructions that node by node takes (8.4k clocks per element on that pipe before)
-        Sum4 V[TY][2], I[2];
-        Sum3 C[TX][2];
+        if constexpr (SH::TPX == 8 && SH::ACT == NT && NST <= 32) {
+            // 5. moments, a lane's nodes 4 x 2 and a warp's 32 x 8: the envelopes' two floats meet in
+            //    error-free FP32 sums, first a lane's, then by a reduce-scatter over the warp -- rows
+            //    (weights in v) and the internal energy over the eight lanes of a row, columns (weights
+            //    in u) over the four lanes of a column -- so that a lane ends with one row or energy sum
+            //    and one column: 12 FP64 instructions a thread instead of 42, for 200 FP32 ones and
+            //    shuffles.  Pays where few states leave the passes short beside the FP64 pipe: curved
+            //    triangles (24 states) 242 -> 224 us a step; with 48 states the passes set the pace and
+            //    the step loses (128^2 P3 2.95 -> 2.99 ms), hence the line between the two
+            LaneSum2 V[2], C[2][2], I[2];   // V: both rows of a lower or upper envelope, C: [pair of columns]
 #pragma unroll
-        for (int s = 0; s < 2; s++) {
+            for (int s = 0; s < 2; s++) {
+                const float2(&M)[TY][2] = s ? thi : tlo;
+                const float2(&r)[TY][2] = s ? eth : etl;
+                const LaneSum2 v0 = lane_pair(M[0][0], r[0][0], M[0][1], r[0][1]);
+                const LaneSum2 v1 = lane_pair(M[1][0], r[1][0], M[1][1], r[1][1]);
+                V[s] = lane_merge(lane_x(v0, v1), lane_y(v0, v1));
+                LaneSum2 ci[2];
 #pragma unroll
-            for (int b = 0; b < TY; b++) {
-                const float2(&M)[2] = s ? thi[b] : tlo[b];
-                const float2(&r)[2] = s ? eth[b] : etl[b];
-                V[b][s] = sum_lanes(sum_pairs(M[0], r[0], M[1], r[1]));
+                for (int p = 0; p < 2; p++) {
+                    C[p][s] = lane_pair(M[0][p], r[0][p], M[1][p], r[1][p]);
+                    ci[p] = s ? lane_pair(ihi[0][p], eih[0][p], ihi[1][p], eih[1][p])
+                              : lane_pair(ilo[0][p], eil[0][p], ilo[1][p], eil[1][p]);
+                }
+                I[s] = lane_merge(ci[0], ci[1]);
             }
-            Sum4x2 ci[2];
-#pragma unroll
-            for (int p = 0; p < 2; p++) {
-                float2 m, e;
-                f2two_sum(s ? thi[0][p] : tlo[0][p], s ? thi[1][p] : tlo[1][p], m, e);
-                const float2 r = __fadd2_rn(s ? eth[0][p] : etl[0][p], s ? eth[1][p] : etl[1][p]);
-                C[2 * p][s] = Sum3{m.x, e.x, r.x};
-                C[2 * p + 1][s] = Sum3{m.y, e.y, r.y};
-                ci[p] = s ? sum_pairs(ihi[0][p], eih[0][p], ihi[1][p], eih[1][p])
-                          : sum_pairs(ilo[0][p], eil[0][p], ilo[1][p], eil[1][p]);
-            }
-            I[s] = sum_lanes(sum_sums(ci[0], ci[1]));
-        }
-        double vs[TY][2];
-#pragma unroll
-        for (int b = 0; b < TY; b++) {
-            const int jy = ty * TY + b;
+            const LaneSum2 both = lane_merge(lane_x(I[0], I[1]), lane_y(I[0], I[1]));
+            // lanes with bit 2: energy, lower or upper by bit 0 (none with bit 1); the others: row bit 0,
+            // lower or upper by bit 1
+            const LaneSum2 none = {f2dup(0.0f), f2dup(0.0f), f2dup(0.0f)};
+            LaneSum2 t = lane_exchange(lane_exchange(V[0], both, lane & 4, 4), lane_exchange(V[1], none, lane & 4, 4),
+                                       lane & 2, 2);
+            t = lane_exchange(t, lane_y(t, t), lane & 1, 1);
+            const bool energy = lane & 4, up = lane & (energy ? 1 : 2);
+            const int jy = ty * TY + (lane & 1);
+            const double val = LaneSum{t.m.x, t.r.x, t.q.x}.value();
             const double v0 = sm.wt[1][0][jy], v1 = sm.wt[1][1][jy], kv = sm.wt[1][2][jy];
-            const bool neg = __double2hiint(v0) < 0;   // v < 0: the lower sum takes the upper envelope
-#pragma unroll
-            for (int s = 0; s < 2; s++) vs[b][s] = V[b][s].value();
-            acc[4] = fma(v0, neg ? vs[b][1] : vs[b][0], acc[4]);
-            acc[5] = fma(v1, neg ? vs[b][0] : vs[b][1], acc[5]);
-            acc[6] = fma(kv, vs[b][0], acc[6]);
-            acc[7] = fma(kv, vs[b][1], acc[7]);
-        }
-        acc[0] = vs[0][0] + vs[1][0];
-        acc[1] = vs[0][1] + vs[1][1];
-        acc[6] += I[0].value();
-        acc[7] += I[1].value();
-#pragma unroll
-        for (int a = 0; a < TX; a++) {
-            const int jx = 4 * tx + a;
+            // v < 0: the lower sum takes the upper envelope
+            const bool lower = up == (__double2hiint(v0) < 0);
+            const double mv = (lower ? v0 : v1) * val, ev = (energy ? (lane & 2 ? 0.0 : 1.0) : kv) * val;
+            acc[0] = energy || up ? 0.0 : val;
+            acc[1] = !energy && up ? val : 0.0;
+            acc[4] = !energy && lower ? mv : 0.0;
+            acc[5] = energy || lower ? 0.0 : mv;
+            // a column's lower and upper sum: column 2 (bit 4) + bit 3 of the lane's four
+            const LaneSum2 c0 = lane_exchange(C[0][0], C[1][0], lane & 16, 16);
+            const LaneSum2 c1 = lane_exchange(C[0][1], C[1][1], lane & 16, 16);
+            const LaneSum2 c = lane_exchange(lane_x(c0, c1), lane_y(c0, c1), lane & 8, 8);
+            const int jx = 4 * tx + ((lane >> 3) & 1) + 2 * (lane >> 4);
+            const double lo = LaneSum{c.m.x, c.r.x, c.q.x}.value(), hi = LaneSum{c.m.y, c.r.y, c.q.y}.value();
             const double u0 = sm.wt[0][0][jx], u1 = sm.wt[0][1][jx], ku = sm.wt[0][2][jx];
             const bool neg = __double2hiint(u0) < 0;
-            const double c0 = C[a][0].value(), c1 = C[a][1].value();
-            acc[2] = fma(u0, neg ? c1 : c0, acc[2]);
-            acc[3] = fma(u1, neg ? c0 : c1, acc[3]);
-            acc[6] = fma(ku, c0, acc[6]);
-            acc[7] = fma(ku, c1, acc[7]);
+            acc[2] = u0 * (neg ? hi : lo);
+            acc[3] = u1 * (neg ? lo : hi);
+            acc[6] = fma(ku, lo, up ? 0.0 : ev);
+            acc[7] = fma(ku, hi, up ? ev : 0.0);
+        } else {
+            // 5. moments: the envelopes' two floats meet in error-free FP32 sums (a row over x for the weights
+            //    in v, a column over y for those in u, everything for I), which then enter FP64: a third of
+            //    the FP64 instructions that node by node takes (8.4k clocks per element on that pipe before)
+            Sum4 V[TY][2], I[2];
+            Sum3 C[TX][2];
+    #pragma unroll
+            for (int s = 0; s < 2; s++) {
+    #pragma unroll
+                for (int b = 0; b < TY; b++) {
+                    const float2(&M)[2] = s ? thi[b] : tlo[b];
+                    const float2(&r)[2] = s ? eth[b] : etl[b];
+                    V[b][s] = sum_lanes(sum_pairs(M[0], r[0], M[1], r[1]));
+                }
+                Sum4x2 ci[2];
+    #pragma unroll
+                for (int p = 0; p < 2; p++) {
+                    float2 m, e;
+                    f2two_sum(s ? thi[0][p] : tlo[0][p], s ? thi[1][p] : tlo[1][p], m, e);
+                    const float2 r = __fadd2_rn(s ? eth[0][p] : etl[0][p], s ? eth[1][p] : etl[1][p]);
+                    C[2 * p][s] = Sum3{m.x, e.x, r.x};
+                    C[2 * p + 1][s] = Sum3{m.y, e.y, r.y};
+                    ci[p] = s ? sum_pairs(ihi[0][p], eih[0][p], ihi[1][p], eih[1][p])
+                              : sum_pairs(ilo[0][p], eil[0][p], ilo[1][p], eil[1][p]);
+                }
+                I[s] = sum_lanes(sum_sums(ci[0], ci[1]));
+            }
+            double vs[TY][2];
+    #pragma unroll
+            for (int b = 0; b < TY; b++) {
+                const int jy = ty * TY + b;
+                const double v0 = sm.wt[1][0][jy], v1 = sm.wt[1][1][jy], kv = sm.wt[1][2][jy];
+                const bool neg = __double2hiint(v0) < 0;   // v < 0: the lower sum takes the upper envelope
+    #pragma unroll
+                for (int s = 0; s < 2; s++) vs[b][s] = V[b][s].value();
+                acc[4] = fma(v0, neg ? vs[b][1] : vs[b][0], acc[4]);
+                acc[5] = fma(v1, neg ? vs[b][0] : vs[b][1], acc[5]);
+                acc[6] = fma(kv, vs[b][0], acc[6]);
+                acc[7] = fma(kv, vs[b][1], acc[7]);
+            }
+            acc[0] = vs[0][0] + vs[1][0];
+            acc[1] = vs[0][1] + vs[1][1];
+            acc[6] += I[0].value();
+            acc[7] += I[1].value();
+    #pragma unroll
+            for (int a = 0; a < TX; a++) {
+                const int jx = 4 * tx + a;
+                const double u0 = sm.wt[0][0][jx], u1 = sm.wt[0][1][jx], ku = sm.wt[0][2][jx];
+                const bool neg = __double2hiint(u0) < 0;
+                const double c0 = C[a][0].value(), c1 = C[a][1].value();
+                acc[2] = fma(u0, neg ? c1 : c0, acc[2]);
+                acc[3] = fma(u1, neg ? c0 : c1, acc[3]);
+                acc[6] = fma(ku, c0, acc[6]);
+                acc[7] = fma(ku, c1, acc[7]);
+            }
         }
     }
     // 6. warp reduce-scatter of the eight sums (lane 4 k holds sum k), then the warps
