@@ -234,7 +234,10 @@ cudaError_t dalloc(T** p, size_t count)
 // both.  Step time against one main chain traces -> residual -> bounds -> stage of programmatic
 // dependents: 200 1D P3 elements in FP64 82 us there, 62 here; 16^2 P3 mixed 51 and 45, 32^2 FP64
 // 274 and 243; at 128^2 the bounds fill the chip and little is left to hide: mixed 515 and 513,
-// FP64 3025 and 3001 (so no rule on the size).
+// FP64 3025 and 3001 (so no rule on the size).  FP32 bounds on more than 32 velocity nodes per axis
+// keep the one chain (ctx->pdl_chain: residuals and stages programmatic dependents as well): their
+// blocks of 256 threads wait for room beside the residual's, and a branch cost more than it hid (200^2
+// P3, 48 nodes: 5.66 ms per step in the chain, 5.83 with the branch).
 int issue_step(kbl_ctx* c, double* w, double cfl, cudaStream_t s, cudaStream_t s2 = nullptr,
                cudaEvent_t* ev = nullptr)
 {
@@ -254,18 +257,22 @@ int issue_step(kbl_ctx* c, double* w, double cfl, cudaStream_t s, cudaStream_t s
     const double* wn = w;
     const double* ws = w;
     double* outs[3] = {c->d_wa, c->d_wb, w};
+    const bool beside = s2 && !c->pdl_chain;
     for (int st = 0; st < 3; st++) {
-        if (s2) {   // the residual on the side branch, behind the traces (stage 0: and the time step)
+        if (beside) {   // the residual on the side branch, behind the traces (stage 0: and the time step)
             if (cudaEventRecord(ev[0], s) != cudaSuccess || cudaStreamWaitEvent(s2, ev[0], 0) != cudaSuccess) return -1;
             if ((r = launch_rhs(c, ws, c->d_wf, c->d_R, s2)) < 0) return -1;
             if (cudaEventRecord(ev[1], s2) != cudaSuccess) return -1;
-        } else if ((r = launch_rhs(c, ws, c->d_wf, c->d_R, s)) < 0) {
-            return -1;
+        } else {
+            if (s2 && st == 0 &&   // the time step joins before the first residual
+                (cudaEventRecord(ev[1], s2) != cudaSuccess || cudaStreamWaitEvent(s, ev[1], 0) != cudaSuccess))
+                return -1;
+            if ((r = launch_rhs(c, ws, c->d_wf, c->d_R, s)) < 0) return -1;
         }
         n += r;
         if ((r = launch_bounds(c, ws, c->d_wf, c->d_bnd, s)) < 0) return -1;
         n += r;
-        if (s2 && cudaStreamWaitEvent(s, ev[1], 0) != cudaSuccess) return -1;
+        if (beside && cudaStreamWaitEvent(s, ev[1], 0) != cudaSuccess) return -1;
         if ((r = launch_stage_step(c, st, wn, ws, c->d_R, c->d_bnd, outs[st], st < 2 ? c->d_wf : nullptr, st == 2, s)) <
             0)
             return -1;
@@ -665,9 +672,11 @@ kbl_status kbl_step(kbl_ctx* c, double* w, double cfl)
             release();
             return cuda_fail(c, e, "begin capture");
         }
+        c->pdl_chain = side && c->cfg.dim == 2 && c->cfg.precision == KBL_FP32_MIXED &&
+                       std::max(c->cfg.nu[0], c->cfg.nu[1]) > 32;
         c->pdl = side != nullptr;   // traces and bounds of the branched graph as programmatic dependents
         const int n = issue_step(c, w, cfl, cap, side, ev);
-        c->pdl = false;
+        c->pdl = c->pdl_chain = false;
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(cap, &g);
         release();

@@ -289,6 +289,7 @@ struct kbl_ctx {
     int overlap_rhs = 1;        // knob: 1 the step graph has a side branch (time step, residuals)
     mutable bool pdl = false;   // set while the branched step graph is captured: its traces and
                                 // bounds are programmatic dependents (kbl_grid_dep_sync)
+    mutable bool pdl_chain = false;   // with pdl: residuals and stages are too, in one chain
     std::string err;
     int64_t launches = 0;
     int bounds_tile = 0;        // FP32 bounds thread tile: 0 = 4x4 nodes, 1 = 4x2 nodes

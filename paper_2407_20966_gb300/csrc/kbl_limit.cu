@@ -54,8 +54,10 @@ k_stage_limit_step(const double* wn, const double* ws, const double* __restrict_
                    int advance, int E, FrOps ops, Phys ph, DevFlags* flags)
 {
     using SH = LimShape<DIM, N>;
-    // the next stage's bounds launch may be its programmatic dependent: that grid waits for this one
-    // before it touches memory
+    // the next launch of the branch may be its programmatic dependent: that grid waits for this one
+    // before it touches memory.  In the one chain this kernel is itself one, of the bounds launch: what
+    // was complete before that launch began (wn, ws, R, dt) it reads at once, the bounds after the wait
+    // in stage_limit_block
     kbl_grid_dep_trigger();
     __shared__ kbl_dev::LimSmem<DIM, N, SH::EPB> sm;
     const double dt = scal[0];
@@ -76,14 +78,14 @@ int run_stage_step(const kbl_ctx* c, int stage, const double* wn, const double* 
     const unsigned grid = (unsigned)((c->E + SH::EPB - 1) / SH::EPB);
     // one kernel per stage: the stage's combination is fixed at compile time
     if (stage == 0)
-        k_stage_limit_step<DIM, N, 0><<<grid, SH::NT, 0, s>>>(wn, ws, R, bnd, c->d_scal, wout, wf_next, advance, c->E,
-                                                            c->ops, c->phys, c->d_flags);
+        kbl_launch(k_stage_limit_step<DIM, N, 0>, grid, SH::NT, 0, s, c->pdl_chain, wn, ws, R, bnd, c->d_scal, wout,
+                   wf_next, advance, c->E, c->ops, c->phys, c->d_flags);
     else if (stage == 1)
-        k_stage_limit_step<DIM, N, 1><<<grid, SH::NT, 0, s>>>(wn, ws, R, bnd, c->d_scal, wout, wf_next, advance, c->E,
-                                                            c->ops, c->phys, c->d_flags);
+        kbl_launch(k_stage_limit_step<DIM, N, 1>, grid, SH::NT, 0, s, c->pdl_chain, wn, ws, R, bnd, c->d_scal, wout,
+                   wf_next, advance, c->E, c->ops, c->phys, c->d_flags);
     else
-        k_stage_limit_step<DIM, N, 2><<<grid, SH::NT, 0, s>>>(wn, ws, R, bnd, c->d_scal, wout, wf_next, advance, c->E,
-                                                            c->ops, c->phys, c->d_flags);
+        kbl_launch(k_stage_limit_step<DIM, N, 2>, grid, SH::NT, 0, s, c->pdl_chain, wn, ws, R, bnd, c->d_scal, wout,
+                   wf_next, advance, c->E, c->ops, c->phys, c->d_flags);
     return 1;
 }
 

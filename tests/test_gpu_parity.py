@@ -583,3 +583,24 @@ def test_step_residual_branch_is_bitwise_serial(orc, precision, dim, p, n, stric
         assert cnt[0]["limited_elements"] > 0 and cnt[0]["pressure_relimits"] > 0   # the exact limiter cut
     for k in cnt[0]:
         np.testing.assert_array_equal(cnt[0][k], cnt[1][k], err_msg=k)
+
+
+@pytest.mark.parametrize("p,nu,quad", [(1, 33, 1), (3, 34, 0), (3, 48, 0), (5, 64, 0)])
+def test_step_one_chain_is_bitwise_serial(orc, p, nu, quad):
+    """FP32 bounds on more than 32 nodes per axis: the step graph is one chain of programmatic
+    dependents, and gives the serial graph's state bit for bit."""
+    from paper_2407_20966_gb300 import kbl
+    ctx, _ = both(orc, 2, p, (nu, nu), precision=1, quadrature=quad)
+    mesh, w = mesh_and_field(orc, 2, p, (13, 11), seed=22, kind="disc", periodic=True)
+    upload(ctx, orc, mesh)
+    out = []
+    for ov in (1, 0):
+        ctx.set_tuning(kbl.TUNE_RHS_OVERLAP, ov)
+        wd = to_dev(w)
+        ctx.set_time(0.0)
+        for _ in range(3):
+            ctx.step(wd, 0.05)
+        ctx.check()
+        out.append((wd.cpu().numpy(), ctx.time()))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    assert out[0][1] == out[1][1] > 0.0
