@@ -295,7 +295,8 @@ typedef enum { KBL_TUNE_BOUNDS_TILE = 0, KBL_TUNE_RHS_TC = 1, KBL_TUNE_RHS_OVERL
 /* KBL_TUNE_RHS_OVERLAP: 1 (default) the step graph has two branches: the time step runs beside
  * the traces and each stage's residual beside its bounds, the stage kernel joins them, and the
  * bounds launch is a programmatic dependent of the stage before it, so that its blocks are in
- * place when that one ends.  0: one ordinary launch after the other.  The same arithmetic runs
+ * place when that one ends (FP32 2D bounds on more than 32 nodes per axis: one chain of
+ * programmatic dependents, the time step on a branch).  0: one ordinary launch after the other.  The same arithmetic runs
  * either way: results are identical.  Setting it drops the captured step graph. */
 kbl_status kbl_set_tuning(kbl_ctx* ctx, int key, int value);   /* KBL_EINVAL for an unknown key or value */
 kbl_status kbl_get_tuning(const kbl_ctx* ctx, int key, int* value);
@@ -365,7 +366,7 @@ kbl_status kbl_batch_bounds_ms(kbl_batch* b, double* ms);
  * in phase order and wait, per problem, only for the earlier phases that problem's item depends
  * on (bounded waits: a wait that runs out raises the timeout flag, which kbl_batch_check
  * reports as KBL_ETIMEOUT, and ends the launch); 0 (default) one persistent launch per phase
- * (14 launches), each in the launch shape the autotuner picks for its phase -- measured about
+ * (13 launches), each in the launch shape the autotuner picks for its phase -- measured about
  * 6% faster on the batched benchmark workload, as the one-launch kernel is compiled for the
  * register budget of its most demanding phase.  Both run the same device code per element:
  * results are identical.  Drops the captured graphs.  KBL_EINVAL for other values. */
