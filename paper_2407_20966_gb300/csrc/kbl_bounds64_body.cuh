@@ -304,10 +304,13 @@ __device__ __forceinline__ void bounds2d_f64_core(Bounds2dF64Smem<NST, NX>& sm, 
 // GB300 runs FP64 at 1.7 lanes per clock per SM and FP32 at 128, so the envelopes of the FP64 mode
 // are formed on unevaluated sums of two floats (hi + lo, 48-49 significant bits) and the FP64 pipe
 // keeps what decides the result's accuracy per state (the primitive state, the velocity box, the
-// exponents' coefficients) and per sum (the moments).  Errors against extended precision (2-norm; the
-// kernel above in brackets, its tables drift along the recurrence): vortex 2.1e-16 (2.8e-16), smooth
-// waves 2.0e-16 (2.6e-16), blast 2.2e-16 (4.4e-16), scattered states 2.1e-16 (2.3e-16), 64 nodes
-// 1.7e-16 (4.4e-16), 33 nodes by Romberg 2.7e-16 (2.6e-16).
+// exponents' coefficients) and per sum (the moments).  Errors against extended precision, every bound
+// relative to itself (a momentum to the magnitudes it sums), rms; the kernel above in brackets, its
+// tables drift along the recurrence: vortex 2.2e-16 (2.5e-16), smooth waves 1.9e-16 (2.4e-16), blast
+// 2.0e-16 (2.6e-16), scattered node sets 2.0e-16 (2.0e-16); blast, 48 nodes 1.8e-16 (2.5e-16), 33 nodes
+// by Romberg 2.3e-16 (2.6e-16).  States that differ by factors within a stencil: lower density and
+// energy 3.3e-16 (1.8e-16), all bounds 2.6e-16 (1.9e-16), since their envelope's minimum lives on few
+// nodes and the tables' 2^-49 average out less.
 //
 //   row tables   a_i(u) = A_i 2^-t(u), c_i = C_i a_i, b_i(v) = 2^-t(v), t = (u - U)^2 log2(e)/(2 theta),
 //                t in 64-bit fixed point by second differences (exact additions), 2^-t by a table of
@@ -485,14 +488,14 @@ __device__ __forceinline__ Triple2 exp2_pair(long long t0, long long t1, const f
     return triple_of(yh, f2sub(w, f2sub(yh, Th)), Tl, we, f2dup(0.0f));
 }
 
-// y scaled by sc (powers of two), rounded to a pair with the rounding error carried into the next
-// entry of the row: the errors of neighbouring entries cancel in the sums over the nodes.
-__device__ __forceinline__ void triple_store(const Triple2& y, float2 sc, float2& carry, float2& h, float2& l)
+// y scaled by sc (powers of two; 0 for a node without weight, whose pair is then 0 and 0).  The third
+// float, at most half a last place of the second, is dropped: handing it on to a later node of the row
+// to even out the row's sum leaves an error of this node's size in one that may be far smaller, where
+// it decides the lower envelope (1e-10 of a lower density across two separated streams).
+__device__ __forceinline__ void triple_store(const Triple2& y, float2 sc, float2& h, float2& l)
 {
     h = __fmul2_rn(y.h, sc);
-    const float2 lt = __fmul2_rn(y.l, sc), rt = __ffma2_rn(y.r, sc, carry);
-    l = __fadd2_rn(lt, rt);
-    carry = f2sub(rt, f2sub(l, lt));
+    l = __fmul2_rn(y.l, sc);
 }
 
 // x in units of 2^-58, rounded; |x| < 32.
@@ -886,7 +889,6 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
         const long long dd = (__mul64hi(8 * dz, 4 * dz) + 1) >> 1;
         if (axis == 0) t += 95530215845326779ll;   // log2(2 pi): the Maxwellian's 1 / (2 pi)
         const Triple A = s.A, C = s.C;
-        float2 ca = f2dup(0.0f), cc = ca;   // rounding errors of the even and the odd nodes
 #pragma unroll 1
         for (int j = jb; j < jb + SEG; j += 2) {
             int n0, n1;
@@ -906,15 +908,15 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
             float2 h, l;
             if (axis == 0) {
                 y = triple_mul(y, f2dup(A.h), f2dup(A.l), f2dup(A.r));
-                triple_store(y, sc, ca, h, l);
+                triple_store(y, sc, h, l);
                 *(float2*)&sm.u.tab.x[i][0][j] = h;
                 *(float2*)&sm.u.tab.x[i][1][j] = l;
                 y = triple_mul(y, f2dup(C.h), f2dup(C.l), f2dup(C.r));
-                triple_store(y, sc, cc, h, l);
+                triple_store(y, sc, h, l);
                 *(float2*)&sm.u.tab.x[i][2][j] = h;
                 *(float2*)&sm.u.tab.x[i][3][j] = l;
             } else {
-                triple_store(y, sc, ca, h, l);
+                triple_store(y, sc, h, l);
                 *(float2*)&sm.u.tab.y[i][0][j] = h;
                 *(float2*)&sm.u.tab.y[i][1][j] = l;
             }
