@@ -113,6 +113,14 @@ struct NodeWeights {
     double w[64];
 };
 
+// Element of a thread, four threads each: up to 2^31 - 1 elements the thread's index takes 33 bits.
+__host__ __device__ constexpr long long node_element(unsigned block, unsigned threads, unsigned thread)
+{
+    return ((long long)block * threads + thread) >> 2;
+}
+static_assert(node_element((1u << 25) - 1u, 128, 127) == (1ll << 30) - 1 && node_element(1u << 25, 128, 0) == 1ll << 30 &&
+              node_element((1u << 26) - 1u, 128, 127) == (1ll << 31) - 1, "the last element of the largest set");
+
 // The node-set limiter, FP64 and the checker's arithmetic.  Of the four threads of an element each
 // takes a component for the mean, the extremes and the limited values (a 32-byte record is read
 // whole) and every fourth point of V for the pressures; the operations per value and their order
@@ -138,8 +146,9 @@ __global__ void __launch_bounds__(128) k_limit_nodes(int E, int ns, int nf, Node
                                                      double* F_out, const double* __restrict__ We)
 {
     constexpr int DIM = NV - 2;
-    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 2, c = threadIdx.x & 3;
-    if (e >= E) return;
+    const long long el = node_element(blockIdx.x, blockDim.x, threadIdx.x);
+    if (el >= E) return;
+    const int e = (int)el, c = threadIdx.x & 3;
     const unsigned four = 0xfu << (threadIdx.x & 28);   // the element's lanes
     double* u = U + (size_t)e * ns * NV;
     const double* f = F + (size_t)e * nf * NV;

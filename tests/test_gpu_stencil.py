@@ -149,3 +149,24 @@ def test_limit_node_sets_argument_checks():
                       (np.ones(6), U, zeros_dev(3, 65, 4))):
         with pytest.raises(kbl.KblError):
             ctx.limit_nodes(W, UU, FF, bnd)
+
+
+def test_limit_node_sets_beyond_2_30_elements():
+    """Single-point node sets of 2^30 + 64 elements: four threads each are more than 2^32 threads,
+    and every element is still limited, by its own four."""
+    import torch
+    from paper_2407_20966_gb300 import kbl
+    E = 2 ** 30 + 64
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info()[0] < 110e9:
+        pytest.skip("needs 95 GB of device memory")
+    ctx = kbl.Context(dim=1, p=2, nu=(64,), eps=0.0)
+    U = torch.tensor([1.0, 0.5, 3.0], dtype=torch.float64, device="cuda").repeat(E, 1).reshape(E, 1, 3)
+    bnd = torch.empty((2, 3, E), dtype=torch.float64, device="cuda")
+    for v, q in enumerate((1.0, 0.5, 3.0)):
+        bnd[0, v], bnd[1, v] = q - 0.1, q + 0.1
+    alpha = torch.full((2, E), 7.0, dtype=torch.float64, device="cuda")
+    ctx.limit_nodes(np.ones(1), U, U[:, :0], bnd, alpha)
+    ctx.check()
+    at = torch.tensor([0, 63, 64, 2 ** 30 - 1, 2 ** 30, E - 1], device="cuda")
+    assert bool((alpha[:, at] == 1.0).all()) and float(alpha.max()) == 1.0
