@@ -1172,7 +1172,7 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
 
 // ---------------------------------------------------------------------------
 // 1D, full precision: every Maxwellian of a node as three floats (exp2_pair on fixed-point
-// exponents), the envelopes by comparing their leading two, the sums in FP64
+// exponents), the envelopes by comparing those, the sums in FP64
 // ---------------------------------------------------------------------------
 // Per-state constants: as PairState, the step in units of 2^-(58 + floor(log2 nu)).
 struct LineState {
@@ -1180,11 +1180,13 @@ struct LineState {
     Triple A, C;
 };
 
-// The larger (UP) or smaller of best and x, decided on the leading two floats.
+// The larger (UP) or smaller of best and x, decided on all three floats: of states equal to 1e-15 or so
+// the leading two cannot tell the extreme one, and the lower bounds came out 3e-16 high, the upper ones
+// as much low.
 template <bool UP>
 __device__ __forceinline__ void triple_extreme(Triple& best, const Triple& x)
 {
-    const float d = __fadd_rn(__fsub_rn(x.h, best.h), __fsub_rn(x.l, best.l));
+    const float d = __fadd_rn(__fsub_rn(x.h, best.h), __fadd_rn(__fsub_rn(x.l, best.l), __fsub_rn(x.r, best.r)));
     if (UP ? d > 0.0f : d < 0.0f) best = x;
 }
 __device__ __forceinline__ double triple_value(const Triple& a)
