@@ -287,7 +287,7 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
             if (axis == 0)
                 kbl_gauss_segment(s.A, s.U[0], s.th, sbox[0], hx, NX, jb, jb + SEG, [&](int j, double v) {
                     sEx[i][j] = v;
-                    sExc[i][j] = s.C * v;
+                    sExc[i][j] = fabs(s.C) * v;
                 });
             else
                 kbl_gauss_segment(1.0, s.U[1], s.th, sbox[2], hy, NX, jb, jb + SEG,
@@ -304,7 +304,8 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
         for (int jj = tid; jj < CHUNK; jj += NT) {
             const int j = c0 + jj, jx = j % NX, jy = j / NX;
             const double ux = sux[jx], uy = suy[jy], M = swx[jx] * swy[jy];
-            // compared as bit patterns: all values are >= +0
+            // compared as bit patterns: all values are >= +0, the internal ones with |C| (C has one sign,
+            // negative for gamma > 2: there the largest |C| g is the lowest C g)
             long long tl = __double_as_longlong(DBL_MAX), th = 0, il = tl, ih = 0;
             int itl = 0, ith = 0, iil = 0, iih = 0;
 #pragma unroll 4
@@ -317,7 +318,13 @@ k_bounds2d_vjp(const double* __restrict__ w, const double* __restrict__ wf, cons
                 if (cg > ih) { ih = cg; iih = i; }
             }
             const double Tl = rm * __longlong_as_double(tl), Th = rp * __longlong_as_double(th);
-            const double Il = rm * __longlong_as_double(il), Ih = rp * __longlong_as_double(ih);
+            if (delta < 0.0) {
+                const int i = iil;
+                iil = iih;
+                iih = i;
+            }
+            const double i0 = __longlong_as_double(il), i1 = __longlong_as_double(ih);
+            const double Il = rm * (delta < 0.0 ? -i1 : i0), Ih = rp * (delta < 0.0 ? -i0 : i1);
             const double ke = 0.5 * (ux * ux + uy * uy);
             const double* lb = sB;
             const double* hb = sB + 4;

@@ -180,7 +180,7 @@ k_bounds1d_f32(const double* __restrict__ w, const double* __restrict__ wf, Mesh
         const double ud = lo + j * h;
         const float u = (float)ud, ur = (float)(ud - c);
         const float q = (float)kbl_qweight(ph, j, NU);
-        float Tl = FLT_MAX, Th = 0.0f, Il = FLT_MAX, Ih = 0.0f;
+        float Tl = FLT_MAX, Th = 0.0f, Il = FLT_MAX, Ih = -FLT_MAX;   // C < 0 for gamma > 3
 #pragma unroll
         for (int i = 0; i < NST; i++) {
             const float d = ur - Ur[i];

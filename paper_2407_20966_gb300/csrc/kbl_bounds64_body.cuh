@@ -148,7 +148,8 @@ __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsig
 // ---------------------------------------------------------------------------
 // 2D, FP64 arithmetic throughout: row tables by the product recurrence of kbl_gauss_segment,
 // products and envelopes in FP64 (min/max as unsigned 64-bit compares of the bit patterns: all
-// values are >= +0, where integer order is value order).  Bound by the FP64 pipe: two products per
+// values are >= +0, where integer order is value order; the internal weights C, of one sign for all
+// states and negative for gamma > 2, enter as |C|).  Bound by the FP64 pipe: two products per
 // (state, node) at 1.7 lanes per clock per SM.  Runs the grids the pairs below do not cover.
 // ---------------------------------------------------------------------------
 template <int NST, int NX, int NW>
@@ -215,7 +216,7 @@ __device__ __forceinline__ void bounds2d_f64_states(const double (*S)[4], F64Tab
             if (axis == 0)
                 kbl_gauss_segment(s.A, s.U[0], s.th, sm.box[0], sm.gh[0], nu, jb, jb + SEG, [&](int j, double v) {
                     sm.ex[i][j] = v;
-                    sm.exc[i][j] = s.C * v;
+                    sm.exc[i][j] = fabs(s.C) * v;
                 });
             else
                 kbl_gauss_segment(1.0, s.U[1], s.th, sm.box[2], sm.gh[1], nu, jb, jb + SEG,
@@ -256,7 +257,9 @@ __device__ __forceinline__ void bounds2d_f64_states(const double (*S)[4], F64Tab
                 const double M = sm.w[0][jx] * sm.w[1][jy];
                 const double ux = sm.u[0][jx], uy = sm.u[1][jy];
                 const double Tl = __longlong_as_double(tlo[a][b]), Th = __longlong_as_double(thi[a][b]);
-                const double Il = __longlong_as_double(ilo[a][b]), Ih = __longlong_as_double(ihi[a][b]);
+                const double i0 = __longlong_as_double(ilo[a][b]), i1 = __longlong_as_double(ihi[a][b]);
+                const bool neg = ph.half_delta2 < 0.0;
+                const double Il = neg ? -i1 : i0, Ih = neg ? -i0 : i1;
                 acc[0] += M * Tl;
                 acc[1] += M * Th;
                 if (ux < 0.0) { acc[2] += M * Th * ux; acc[3] += M * Tl * ux; }
@@ -1219,7 +1222,7 @@ __device__ __noinline__ LineSums bounds1d_f64_nodes(const StatePrim* sP, const P
     for (int k = 0; k < 8; k++) s.v[k] = 0.0;
     for (int j = tid; j < ph.nu[0]; j += nt) {
         const double u = lo + j * h, q = kbl_qweight(ph, j, ph.nu[0]);
-        double Tl = DBL_MAX, Th = 0.0, Il = DBL_MAX, Ih = 0.0;
+        double Tl = DBL_MAX, Th = 0.0, Il = DBL_MAX, Ih = -DBL_MAX;
         for (int i = 0; i < NST; i++) {
             const double d = u - sP[i].U[0];
             const double g = sP[i].A * exp(-(d * d) / (2.0 * sP[i].th));

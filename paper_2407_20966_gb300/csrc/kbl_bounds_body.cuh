@@ -351,7 +351,7 @@ __device__ __forceinline__ void bounds2d_f32_core(Bounds2dF32SmemS<NST_, NX, TYS
 #pragma unroll
         for (int b = 0; b < TY; b++) {
             tlo[a][b] = FLT_MAX; ilo[a][b] = FLT_MAX;
-            thi[a][b] = 0.0f; ihi[a][b] = 0.0f;
+            thi[a][b] = 0.0f; ihi[a][b] = -FLT_MAX;   // C < 0 for gamma > 2
         }
     // unroll factor by pair count, measured (fractions of the envelope-pattern peak on the bench
     // workloads): 12 for 24 or 48 pairs (P3 quads: 0.676 against 0.669 at 8), 4 for odd counts
