@@ -356,35 +356,33 @@ __device__ __forceinline__ void tri_common_flux(const T* qi, const T* qe, T nx, 
     F[3] = Fl[3];
 }
 
-template <typename T>
-__device__ __forceinline__ T tri_in(double x) { return kbl_dev::from_f64<T>(x); }
+__device__ __forceinline__ float tri_in(double x) { return kbl_dev::from_f64<float>(x); }
 
 // The mixed precision's residual: one thread per element, order P fixed at compile time (the loops
-// unroll, the fluxes stay in registers), FP32 arithmetic T on FP64 storage.  The
+// unroll, the fluxes stay in registers), FP32 arithmetic on FP64 storage.  The
 // physical fluxes enter as contravariant fluxes Fr = (dr/dx) Fx + (dr/dy) Fy, Fs = (ds/dx) Fx +
 // (ds/dy) Fy, so that -div F_h(x_i) = -sum_j (dr_ij Fr_j + ds_ij Fs_j); the normal flux at a flux
 // point is a_f Fr_h + b_f Fs_h with (a_f, b_f) = J^T n_f of its edge; the jump of the common flux
 // is lifted with lift_qi |e_f| / det J.
-template <int P, typename T>
+template <int P>
 __global__ void __launch_bounds__(128) k_tri_rhs(const double* __restrict__ w, const double* __restrict__ wf,
                                                  TriMeshDev m, TriOps o, double gamma_d, int flux,
                                                  double* __restrict__ R)
 {
-    constexpr bool F32 = sizeof(T) == sizeof(float);
     constexpr int ns = (P + 1) * (P + 2) / 2, nfp = 3 * (P + 1);
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= m.E) return;
     const TriGeo& g = m.geo[e];
-    const T rx = tri_in<T>(g.rx), ry = tri_in<T>(g.ry), sx = tri_in<T>(g.sx), sy = tri_in<T>(g.sy);
-    const T gamma = tri_in<T>(gamma_d), gm1 = F32 ? gamma - T(1) : tri_in<T>(gamma_d - 1.0);
-    T Fr[ns][4], Fs[ns][4], out[ns][4];
+    const float rx = tri_in(g.rx), ry = tri_in(g.ry), sx = tri_in(g.sx), sy = tri_in(g.sy);
+    const float gamma = tri_in(gamma_d), gm1 = gamma - 1.0f;
+    float Fr[ns][4], Fs[ns][4], out[ns][4];
 #pragma unroll
     for (int j = 0; j < ns; j++) {
-        T q[4], Fx[4], Fy[4];
+        float q[4], Fx[4], Fy[4];
 #pragma unroll
-        for (int v = 0; v < 4; v++) q[v] = tri_in<T>(w[((size_t)e * ns + j) * 4 + v]);
-        kbl_flux<2, T>(q, 0, gm1, Fx);
-        kbl_flux<2, T>(q, 1, gm1, Fy);
+        for (int v = 0; v < 4; v++) q[v] = tri_in(w[((size_t)e * ns + j) * 4 + v]);
+        kbl_flux<2, float>(q, 0, gm1, Fx);
+        kbl_flux<2, float>(q, 1, gm1, Fy);
 #pragma unroll
         for (int v = 0; v < 4; v++) {
             Fr[j][v] = rx * Fx[v] + ry * Fy[v];
@@ -395,83 +393,82 @@ __global__ void __launch_bounds__(128) k_tri_rhs(const double* __restrict__ w, c
     for (int i = 0; i < ns; i++)
 #pragma unroll
         for (int v = 0; v < 4; v++) {
-            T div = T(0);
+            float div = 0.0f;
 #pragma unroll
             for (int j = 0; j < ns; j++) {
-                const T dr = F32 ? (T)o.drf[i][j] : (T)o.dr[i][j];
-                const T ds = F32 ? (T)o.dsf[i][j] : (T)o.ds[i][j];
+                const float dr = o.drf[i][j];
+                const float ds = o.dsf[i][j];
                 div += dr * Fr[j][v] + ds * Fs[j][v];
             }
             out[i][v] = -div;
         }
     // J = inverse of ((rx, ry), (sx, sy)): J00 = x_r = sy det, J01 = x_s = -ry det, J10 = y_r = -sx det,
     // J11 = y_s = rx det
-    const T det = tri_in<T>(g.det);
+    const float det = tri_in(g.det);
 #pragma unroll 1
     for (int f = 0; f < 3; f++) {
-        const T nx = tri_in<T>(g.nx[f]), ny = tri_in<T>(g.ny[f]);
-        const T a = det * (sy * nx - sx * ny), b = det * (rx * ny - ry * nx);
-        const T sc = tri_in<T>(g.len[f]) / det;
+        const float nx = tri_in(g.nx[f]), ny = tri_in(g.ny[f]);
+        const float a = det * (sy * nx - sx * ny), b = det * (rx * ny - ry * nx);
+        const float sc = tri_in(g.len[f]) / det;
 #pragma unroll
         for (int k = 0; k <= P; k++) {
             const int q = f * (P + 1) + k;
-            T qi[4], qe[4], Fc[4];
+            float qi[4], qe[4], Fc[4];
             const double* ext = tri_exterior(m, wf, e, f, k);
 #pragma unroll
             for (int v = 0; v < 4; v++) {
-                qi[v] = tri_in<T>(wf[((size_t)e * nfp + q) * 4 + v]);
-                qe[v] = tri_in<T>(ext[v]);
+                qi[v] = tri_in(wf[((size_t)e * nfp + q) * 4 + v]);
+                qe[v] = tri_in(ext[v]);
             }
-            tri_common_flux<T>(qi, qe, nx, ny, gamma, flux, Fc);
+            tri_common_flux<float>(qi, qe, nx, ny, gamma, flux, Fc);
 #pragma unroll
             for (int v = 0; v < 4; v++) {
-                T fr = T(0), fs = T(0);
+                float fr = 0.0f, fs = 0.0f;
 #pragma unroll
                 for (int j = 0; j < ns; j++) {
-                    const T ph = F32 ? (T)o.phiff[q][j] : (T)o.phif[q][j];
+                    const float ph = o.phiff[q][j];
                     fr += ph * Fr[j][v];
                     fs += ph * Fs[j][v];
                 }
-                const T jump = sc * (Fc[v] - (a * fr + b * fs));
+                const float jump = sc * (Fc[v] - (a * fr + b * fs));
 #pragma unroll
-                for (int i = 0; i < ns; i++) out[i][v] -= (F32 ? (T)o.liftf[q][i] : (T)o.lift[q][i]) * jump;
+                for (int i = 0; i < ns; i++) out[i][v] -= o.liftf[q][i] * jump;
             }
         }
     }
 #pragma unroll
     for (int i = 0; i < ns; i++)
 #pragma unroll
-        for (int v = 0; v < 4; v++) R[((size_t)e * ns + i) * 4 + v] = kbl_dev::to_f64<T>(out[i][v]);
+        for (int v = 0; v < 4; v++) R[((size_t)e * ns + i) * 4 + v] = kbl_dev::to_f64<float>(out[i][v]);
 }
 
-// The residual on curved elements (transformed-flux form): with adj J = |J| J^-1 at each
+// The mixed precision's residual on curved elements (transformed-flux form): with adj J = |J| J^-1 at each
 // solution point, Ft = adj J F; at each flux point the physical unit normal n and the stretch
 // sigma = |dx/dt| / |dxi/dt| of its edge; nh the reference edge's unit normal, L its length:
 //   R_i = -(1/|J_i|) [ sum_j (Dr_ij Ft_r,j + Ds_ij Ft_s,j)
 //                      + sum_q phi_i(x_q) gw_q L / (2 w_i) (sigma_q F*_n,q - (Ft_h . nh)(x_q)) ].
 // One thread per element, as the affine kernel.
-template <int P, typename T>
+template <int P>
 __global__ void __launch_bounds__(128) k_tri_rhs_curved(const double* __restrict__ w, const double* __restrict__ wf,
                                                         TriMeshDev m, TriOps o, double gamma_d, int flux,
                                                         double* __restrict__ R)
 {
-    constexpr bool F32 = sizeof(T) == sizeof(float);
     constexpr int ns = (P + 1) * (P + 2) / 2, nfp = 3 * (P + 1);
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= m.E) return;
     const double* pj = m.pj + (size_t)e * ns * 5;
     const double* fq = m.fq + (size_t)e * nfp * 3;
-    const T gamma = tri_in<T>(gamma_d), gm1 = F32 ? gamma - T(1) : tri_in<T>(gamma_d - 1.0);
-    T Fr[ns][4], Fs[ns][4], acc[ns][4];
+    const float gamma = tri_in(gamma_d), gm1 = gamma - 1.0f;
+    float Fr[ns][4], Fs[ns][4], acc[ns][4];
 #pragma unroll
     for (int j = 0; j < ns; j++) {
-        T q[4], Fx[4], Fy[4];
+        float q[4], Fx[4], Fy[4];
 #pragma unroll
-        for (int v = 0; v < 4; v++) q[v] = tri_in<T>(w[((size_t)e * ns + j) * 4 + v]);
-        kbl_flux<2, T>(q, 0, gm1, Fx);
-        kbl_flux<2, T>(q, 1, gm1, Fy);
-        const T a0 = tri_in<T>(pj[j * 5 + 0]), a1 = tri_in<T>(pj[j * 5 + 1]);
-        const T a2 = tri_in<T>(pj[j * 5 + 2]), a3 = tri_in<T>(pj[j * 5 + 3]);
+        for (int v = 0; v < 4; v++) q[v] = tri_in(w[((size_t)e * ns + j) * 4 + v]);
+        kbl_flux<2, float>(q, 0, gm1, Fx);
+        kbl_flux<2, float>(q, 1, gm1, Fy);
+        const float a0 = tri_in(pj[j * 5 + 0]), a1 = tri_in(pj[j * 5 + 1]);
+        const float a2 = tri_in(pj[j * 5 + 2]), a3 = tri_in(pj[j * 5 + 3]);
 #pragma unroll
         for (int v = 0; v < 4; v++) {
             Fr[j][v] = a0 * Fx[v] + a1 * Fy[v];
@@ -482,11 +479,11 @@ __global__ void __launch_bounds__(128) k_tri_rhs_curved(const double* __restrict
     for (int i = 0; i < ns; i++)
 #pragma unroll
         for (int v = 0; v < 4; v++) {
-            T div = T(0);
+            float div = 0.0f;
 #pragma unroll
             for (int j = 0; j < ns; j++) {
-                const T dr = F32 ? (T)o.drf[i][j] : (T)o.dr[i][j];
-                const T ds = F32 ? (T)o.dsf[i][j] : (T)o.ds[i][j];
+                const float dr = o.drf[i][j];
+                const float ds = o.dsf[i][j];
                 div += dr * Fr[j][v] + ds * Fs[j][v];
             }
             acc[i][v] = div;
@@ -494,41 +491,41 @@ __global__ void __launch_bounds__(128) k_tri_rhs_curved(const double* __restrict
 #pragma unroll 1
     for (int f = 0; f < 3; f++) {
         // reference edges: (0,0)->(1,0), (1,0)->(0,1), (0,1)->(0,0); unit normals and lengths
-        const T nhx = f == 0 ? T(0) : (f == 1 ? T(0.70710678118654752) : T(-1));
-        const T nhy = f == 0 ? T(-1) : (f == 1 ? T(0.70710678118654752) : T(0));
-        const T L = f == 1 ? T(1.4142135623730951) : T(1);
+        const float nhx = f == 0 ? 0.0f : (f == 1 ? 0.70710678118654752f : -1.0f);
+        const float nhy = f == 0 ? -1.0f : (f == 1 ? 0.70710678118654752f : 0.0f);
+        const float L = f == 1 ? 1.4142135623730951f : 1.0f;
 #pragma unroll
         for (int k = 0; k <= P; k++) {
             const int q = f * (P + 1) + k;
-            const T nx = tri_in<T>(fq[q * 3 + 0]), ny = tri_in<T>(fq[q * 3 + 1]), sig = tri_in<T>(fq[q * 3 + 2]);
-            T qi[4], qe[4], Fc[4];
+            const float nx = tri_in(fq[q * 3 + 0]), ny = tri_in(fq[q * 3 + 1]), sig = tri_in(fq[q * 3 + 2]);
+            float qi[4], qe[4], Fc[4];
             const double* ext = tri_exterior(m, wf, e, f, k);
 #pragma unroll
             for (int v = 0; v < 4; v++) {
-                qi[v] = tri_in<T>(wf[((size_t)e * nfp + q) * 4 + v]);
-                qe[v] = tri_in<T>(ext[v]);
+                qi[v] = tri_in(wf[((size_t)e * nfp + q) * 4 + v]);
+                qe[v] = tri_in(ext[v]);
             }
-            tri_common_flux<T>(qi, qe, nx, ny, gamma, flux, Fc);
+            tri_common_flux<float>(qi, qe, nx, ny, gamma, flux, Fc);
 #pragma unroll
             for (int v = 0; v < 4; v++) {
-                T fr = T(0), fs = T(0);
+                float fr = 0.0f, fs = 0.0f;
 #pragma unroll
                 for (int j = 0; j < ns; j++) {
-                    const T ph = F32 ? (T)o.phiff[q][j] : (T)o.phif[q][j];
+                    const float ph = o.phiff[q][j];
                     fr += ph * Fr[j][v];
                     fs += ph * Fs[j][v];
                 }
-                const T jump = L * (sig * Fc[v] - (nhx * fr + nhy * fs));
+                const float jump = L * (sig * Fc[v] - (nhx * fr + nhy * fs));
 #pragma unroll
-                for (int i = 0; i < ns; i++) acc[i][v] += (F32 ? (T)o.liftf[q][i] : (T)o.lift[q][i]) * jump;
+                for (int i = 0; i < ns; i++) acc[i][v] += o.liftf[q][i] * jump;
             }
         }
     }
 #pragma unroll
     for (int i = 0; i < ns; i++) {
-        const T det = tri_in<T>(pj[i * 5 + 4]);
+        const float det = tri_in(pj[i * 5 + 4]);
 #pragma unroll
-        for (int v = 0; v < 4; v++) R[((size_t)e * ns + i) * 4 + v] = kbl_dev::to_f64<T>(-acc[i][v] / det);
+        for (int v = 0; v < 4; v++) R[((size_t)e * ns + i) * 4 + v] = kbl_dev::to_f64<float>(-acc[i][v] / det);
     }
 }
 
@@ -999,12 +996,12 @@ kbl_status tri_residual_on(kbl_tri* t, const double* w, const double* wf, double
             else if (t->curved) run_tri_rhs_f64<2, true>(t, w, wf, R, s);
             else run_tri_rhs_f64<2, false>(t, w, wf, R, s);
         } else if (t->curved) {
-            if (p == 1) k_tri_rhs_curved<1, float><<<grid, 128, 0, s>>>(w, wf, md, t->ops, gam, fl, R);
-            else k_tri_rhs_curved<2, float><<<grid, 128, 0, s>>>(w, wf, md, t->ops, gam, fl, R);
+            if (p == 1) k_tri_rhs_curved<1><<<grid, 128, 0, s>>>(w, wf, md, t->ops, gam, fl, R);
+            else k_tri_rhs_curved<2><<<grid, 128, 0, s>>>(w, wf, md, t->ops, gam, fl, R);
         } else if (p == 1) {
-            k_tri_rhs<1, float><<<grid, 128, 0, s>>>(w, wf, md, t->ops, gam, fl, R);
+            k_tri_rhs<1><<<grid, 128, 0, s>>>(w, wf, md, t->ops, gam, fl, R);
         } else {
-            k_tri_rhs<2, float><<<grid, 128, 0, s>>>(w, wf, md, t->ops, gam, fl, R);
+            k_tri_rhs<2><<<grid, 128, 0, s>>>(w, wf, md, t->ops, gam, fl, R);
         }
     }
     const cudaError_t e = cudaGetLastError();
