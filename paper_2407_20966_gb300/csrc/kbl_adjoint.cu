@@ -113,7 +113,7 @@ k_rhs_vjp(const double* __restrict__ w, const double* __restrict__ wf, const dou
             qr[k2] = side ? qe : qi;
             Fb[k2] = k2 == 1 ? (dir ? Jb[2] : Jb[1]) : k2 == 2 ? (dir ? Jb[1] : Jb[2]) : Jb[k2];
         }
-        rusanov_vjp<2, 0>(ql, qr, gamma, Fb, qlb, qrb);
+        rusanov_vjp<2>(ql, qr, gamma, Fb, qlb, qrb);
         double qib[NV], qeb[NV];
 #pragma unroll
         for (int v = 0; v < NV; v++) {

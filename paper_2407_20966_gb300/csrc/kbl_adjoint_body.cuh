@@ -52,15 +52,15 @@ __device__ __forceinline__ void flux_vjp(const double* q, double gamma, const do
     qb[DIM + 1] += fe * gamma * ud;
 }
 
-// Davis wavespeed |u_D| + c of one state, c = sqrt(gamma P / rho) (the forward expression).
-template <int DIM, int D>
+// Davis wavespeed |u_x| + c of one state along x, c = sqrt(gamma P / rho) (the forward expression).
+template <int DIM>
 __device__ __forceinline__ double wavespeed(const double* q, double gamma)
 {
-    return fabs(q[1 + D] / q[0]) + sqrt(gamma * kbl_pressure<DIM>(q, gamma - 1.0) / q[0]);
+    return fabs(q[1] / q[0]) + sqrt(gamma * kbl_pressure<DIM>(q, gamma - 1.0) / q[0]);
 }
 
-// qb += sb * d(|u_D| + c)/dq; u_D = 0 takes the + branch.
-template <int DIM, int D>
+// qb += sb * d(|u_x| + c)/dq; u_x = 0 takes the + branch.
+template <int DIM>
 __device__ __forceinline__ void wavespeed_vjp(const double* q, double gamma, double sb, double* qb)
 {
     const double gm1 = gamma - 1.0;
@@ -69,11 +69,10 @@ __device__ __forceinline__ void wavespeed_vjp(const double* q, double gamma, dou
     const double uu = u0 * u0 + u1 * u1;
     const double P = gm1 * (q[DIM + 1] - 0.5 * rho * uu);
     const double c = sqrt(gamma * P * inv);
-    const double ud = D == 0 ? u0 : u1;
-    const double sgn = ud < 0.0 ? -1.0 : 1.0;
-    // |u_D|
-    qb[0] += sb * sgn * (-ud * inv);
-    qb[1 + D] += sb * sgn * inv;
+    const double sgn = u0 < 0.0 ? -1.0 : 1.0;
+    // |u_x|
+    qb[0] += sb * sgn * (-u0 * inv);
+    qb[1] += sb * sgn * inv;
     // c: dc = gamma / (2 c rho) (dP - P/rho drho)
     const double f = sb * gamma / (2.0 * c * rho);
     qb[0] += f * (0.5 * gm1 * uu - P * inv);
@@ -82,15 +81,16 @@ __device__ __forceinline__ void wavespeed_vjp(const double* q, double gamma, dou
     qb[DIM + 1] += f * gm1;
 }
 
-// Rusanov flux F = 1/2 (F(ql) + F(qr)) - 1/2 lam (qr - ql), lam = max(s_l, s_r) (Davis):
-// qlb, qrb += its transposed Jacobian applied to Fb.  Ties of the max take the left state.
-template <int DIM, int D>
+// Rusanov flux along x, F = 1/2 (F(ql) + F(qr)) - 1/2 lam (qr - ql), lam = max(s_l, s_r) (Davis):
+// qlb, qrb += its transposed Jacobian applied to Fb (for a y face the caller exchanges the momenta).
+// Ties of the max take the left state.
+template <int DIM>
 __device__ __forceinline__ void rusanov_vjp(const double* ql, const double* qr, double gamma, const double* Fb,
                                             double* qlb, double* qrb)
 {
     constexpr int NV = DIM + 2;
-    const double sl = wavespeed<DIM, D>(ql, gamma);
-    const double sr = wavespeed<DIM, D>(qr, gamma);
+    const double sl = wavespeed<DIM>(ql, gamma);
+    const double sr = wavespeed<DIM>(qr, gamma);
     const double lam = fmax(sl, sr);
     double half[NV], lamb = 0.0;
 #pragma unroll
@@ -100,10 +100,10 @@ __device__ __forceinline__ void rusanov_vjp(const double* ql, const double* qr, 
         qlb[v] += 0.5 * lam * Fb[v];
         lamb += -0.5 * (qr[v] - ql[v]) * Fb[v];
     }
-    flux_vjp<DIM, D>(ql, gamma, half, qlb);
-    flux_vjp<DIM, D>(qr, gamma, half, qrb);
-    if (sl >= sr) wavespeed_vjp<DIM, D>(ql, gamma, lamb, qlb);
-    else wavespeed_vjp<DIM, D>(qr, gamma, lamb, qrb);
+    flux_vjp<DIM, 0>(ql, gamma, half, qlb);
+    flux_vjp<DIM, 0>(qr, gamma, half, qrb);
+    if (sl >= sr) wavespeed_vjp<DIM>(ql, gamma, lamb, qlb);
+    else wavespeed_vjp<DIM>(qr, gamma, lamb, qrb);
 }
 
 // qb += Pb * dP/dq, P = (gamma - 1)(E - |m|^2 / (2 rho)).
