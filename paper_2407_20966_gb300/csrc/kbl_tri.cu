@@ -676,6 +676,7 @@ struct kbl_tri {
     kbl_ctx* ctx = nullptr;     // bounds of explicit stencils and node-set limiting
     TriOps ops;
     int E = 0, n_bc = 0;
+    int nsm = 0;                // the device's SMs
     cudaStream_t stream = nullptr;
     TriGeo* d_geo = nullptr;
     bool curved = false;
@@ -725,10 +726,12 @@ namespace {
 template <int P, bool CURVED>
 void run_tri_rhs_f64(const kbl_tri* t, const double* w, const double* wf, double* R, cudaStream_t s)
 {
-    // 16 elements fill 5 warps at the flux points; meshes that would leave SMs without a block of
-    // 16 take 8 per block (3 warps)
+    // 16 elements of P2 have flux points for 144 of 160 threads, 8 for 72 of 96; but a mesh of up to two
+    // blocks of 16 per SM is over no later with the shorter blocks of 8.  Launch on 152 SMs with 8 / 16,
+    // curved P2: 1,152 elements 16.7 / 19.0 us, 3,528 28.9 / 31.1, 5,000 41.3 / 43.4, 7,200 49.5 / 43.4,
+    // 18,432 124 / 109, 100,352 632 / 569; affine P1: 1,152 12.7 / 12.8, 5,000 23.0 / 23.0, 18,432 66 / 54.
     const TriMeshDev md = tri_dev(t);
-    if (t->E > 16 * 2 * 152)
+    if (t->E > 16 * 2 * t->nsm)
         k_tri_rhs_f64<P, CURVED, 16><<<blocks_for(t->E, 16), 160, 0, s>>>(w, wf, md, t->ops, t->cfg.gamma, t->cfg.flux, R);
     else
         k_tri_rhs_f64<P, CURVED, 8><<<blocks_for(t->E, 8), 96, 0, s>>>(w, wf, md, t->ops, t->cfg.gamma, t->cfg.flux, R);
@@ -811,6 +814,9 @@ kbl_status tri_create(kbl_tri** out, const kbl_config* cfg, int n_elem, const do
         delete t;
         return st;
     }
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&t->nsm, cudaDevAttrMultiProcessorCount, dev);
     FrOps gl;
     kbl_build_fr_ops(cfg->p, gl);
     if (!build_tri_ops(cfg->p, gl, t->ops)) {
