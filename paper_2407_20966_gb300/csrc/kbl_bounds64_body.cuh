@@ -310,7 +310,7 @@ __device__ __forceinline__ void bounds2d_f64_core(Bounds2dF64Smem<NST, NX>& sm, 
 // exponents' coefficients) and per sum (the moments).  Errors against extended precision, every bound
 // relative to itself (a momentum to the magnitudes it sums), rms; the kernel above in brackets, its
 // tables drift along the recurrence: vortex 2.2e-16 (2.5e-16), smooth waves 1.9e-16 (2.4e-16), blast
-// 2.0e-16 (2.6e-16), scattered node sets 2.0e-16 (2.0e-16); blast, 48 nodes 1.8e-16 (2.5e-16), 33 nodes
+// 2.0e-16 (2.6e-16), scattered node sets 2.0e-16 (2.1e-16); blast, 48 nodes 1.7e-16 (2.3e-16), 33 nodes
 // by Romberg 2.3e-16 (2.6e-16).  States that differ by factors within a stencil: lower density and
 // energy 3.3e-16 (1.8e-16), all bounds 2.6e-16 (1.9e-16), since their envelope's minimum lives on few
 // nodes and the tables' 2^-49 average out less.
@@ -523,6 +523,13 @@ __device__ __forceinline__ double quotient_of(double a, double b, double inv)
 {
     const double t = a * inv;
     return fma(fma(-t, b, a), inv, t);
+}
+
+// sqrt(x) from rs = rsqrt(x): one step of Heron's (Newton's) iteration on x rs, its residual by an FMA.
+__device__ __forceinline__ double sqrt_of(double x, double rs)
+{
+    const double s = x * rs;
+    return fma(fma(-s, s, x), 0.5 * rs, s);
 }
 
 // What rs = rsqrt(x), rounded, misses of 1 / sqrt(x).
@@ -763,8 +770,7 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
             U[0] = over_rho(mx);
             U[1] = over_rho(my);
             rs = rsqrt(th);
-            double sq = th * rs;
-            sq = fma(fma(-sq, sq, th), 0.5 * rs, sq);
+            double sq = sqrt_of(th, rs);
             const double it = rs * rs;
             A = rho * it;                           // rho / theta (1 / (2 pi) is in the exponents)
             A = fma(fma(-A, th, rho), it, A);
@@ -1280,8 +1286,7 @@ __device__ __forceinline__ void bounds1d_core(Bounds1dSmem<NST, NT>& sm, int E, 
                 out_of_range = 1;
             }
             rs = rsqrt(th);
-            double sq = th * rs;
-            sq = fma(fma(-sq, sq, th), 0.5 * rs, sq);
+            double sq = sqrt_of(th, rs);
             klo = key64(fma(-ph.k, sq, U));
             khi = key64(fma(ph.k, sq, U));
         }
@@ -1446,11 +1451,19 @@ void kbl_launch_dyn(void (*kernel)(KArgs...), int grid, int block, cudaStream_t 
 
 }  // namespace kbl_dev
 
-// Whether a grid of nu nodes per axis over k thermal units either side runs on float pairs: with 3.75
-// or more nodes per thermal unit the roundings of the pairs (2^-48 per node) average out below the
-// FP64 kernel's error; on coarser grids they do not (16 nodes, k = 4: 3.6e-16 against 1.8e-16,
-// 48 nodes, k = 8: 2.7e-16 against 2.2e-16, 32 nodes, k = 4: 2.2e-16 against 2.3e-16), and the FP64
-// kernel runs, on a tile that holds the grid.
+// Whether a grid of nu nodes per axis over k thermal units either side runs on float pairs: where their
+// errors are no larger than the FP64 kernel's.  A pair's rounding (2^-49 per table entry) averages out
+// over the nodes, so the density of the grid decides; the FP64 kernel's tables drift along their
+// recurrence, over 16 nodes on its tiles of 32 and more but over 8 on that of 24.  Error of every bound
+// relative to itself, rms over vortex, wave, blast, shock-vortex and node-set stencils, pairs / FP64, in
+// units of 1e-16:
+//   nodes per thermal unit  3.6 (30 nodes, k = 4) 2.1 / 2.0, 2.9 (48, 8) 2.4 / 2.1, 3.55 (33 Romberg, 4.5)
+//                           2.6 / 2.3; at the line 3.75 (31, 4) 2.0 / 2.3, 3.8 (40, 5.2) 2.1 / 2.3; above
+//                           it 3.9 (32, 4) 2.0 / 2.5, 4 (33 Romberg, 4) 2.4 / 2.6, 5.9 (48, 4) 1.8 / 2.4
+//   24 nodes and fewer      24, k = 3 2.0 / 1.4; 24, 2 1.8 / 1.5; 20, 2.5 2.1 / 1.5; 17 Romberg, 2 2.6 / 1.9;
+//                           25 nodes, k = 3 1.9 / 2.0
+// Launch at 48 states, 8,192 elements, pairs / FP64: 32 nodes 0.42 / 3.3 ms, 24 nodes 0.42 / 2.6,
+// 40 nodes 0.84 / 8.4, 48 nodes 1.4 / 8.1.
 inline bool kbl_pair_grid(int nu, double k) { return nu - 1 >= 7.5 * k && nu > 24; }
 
 // Run a statement with NX the smallest tile that holds NU nodes per axis: of the pair kernels, or of
