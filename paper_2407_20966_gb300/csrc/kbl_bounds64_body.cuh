@@ -1031,15 +1031,16 @@ __device__ __forceinline__ void bounds2d_pair_core(Bounds2dPairSmem<NST, NX>& sm
             }
         }
 
-        if constexpr (SH::TPX == 8 && SH::ACT == NT && NST <= 32) {
+        if constexpr (SH::TPX == 8 && SH::ACT == NT && NST <= 40) {
             // 5. moments, a lane's nodes 4 x 2 and a warp's 32 x 8: the envelopes' two floats meet in
             //    error-free FP32 sums, first a lane's, then by a reduce-scatter over the warp -- rows
             //    (weights in v) and the internal energy over the eight lanes of a row, columns (weights
             //    in u) over the four lanes of a column -- so that a lane ends with one row or energy sum
             //    and one column: 12 FP64 instructions a thread instead of 42, for 200 FP32 ones and
-            //    shuffles.  Pays where few states leave the passes short beside the FP64 pipe: curved
-            //    triangles (24 states) 242 -> 224 us a step; with 48 states the passes set the pace and
-            //    the step loses (128^2 P3 2.95 -> 2.99 ms), hence the line between the two
+            //    shuffles.  Pays where few states leave the passes short beside the FP64 pipe.  Launch with
+            //    it / without, 16,384 elements: 16 states 421 / 471 us, 20 (P1 quads) 500 / 516, 24 531 / 552,
+            //    33 (P2 quads) 676 / 711; 48 states 844 / 826 (P3 quads 846 / 830): the passes set the pace,
+            //    and the line lies between the two
             LaneSum2 V[2], C[2][2], I[2];   // V: both rows of a lower or upper envelope, C: [pair of columns]
 #pragma unroll
             for (int s = 0; s < 2; s++) {
