@@ -60,10 +60,19 @@ typedef enum {
 } kbl_status;
 
 /* Arithmetic of the path.
- * KBL_FP64: everything in FP64; the 2D bounds on grids of at least 3.75 velocity nodes per thermal
- *   unit ((nu - 1) / (2 k), more than 24 nodes) form the Maxwellians and their envelopes on
- *   unevaluated sums of two FP32 numbers (48 bits) from FP64 states and sum them in FP64, with an
- *   error no larger than FP64 products give (2-norm 2e-16 to 2.5e-16 against extended precision).
+ * KBL_FP64: everything in FP64 but the Maxwellians of the bounds and their envelopes, which are formed
+ *   on unevaluated sums of FP32 numbers from FP64 states and summed in FP64:
+ *   2D, grids of at least 3.75 velocity nodes per thermal unit ((nu - 1) / (2 k)) and more than 24
+ *   nodes: two FP32 numbers (49 bits).  Error of every bound relative to itself (a momentum to the sum
+ *   of its terms' magnitudes), rms: below 3e-16 for smooth fields, blasts and moderately scattered
+ *   states (1.7e-16 to 2.7e-16 measured; 1.9e-16 to 3.8e-16 with FP64 products); below 4.5e-16 where
+ *   the states of a stencil differ by factors (lower density and energy 3.3e-16 on 32 nodes, 3.8e-16
+ *   on 33 with Romberg weights; with FP64 products 1.8e-16 and 2.0e-16).  The lower bounds of states
+ *   far apart in velocity carry the roundings of the states times the Maxwellians' exponents, as they
+ *   do with FP64 products (5e-15 where the lower density is 1e-9 of the upper).  Elements whose lower
+ *   density sum is below 2^-40 of the largest state's, or whose states leave the FP32 exponents inside
+ *   the box (a temperature ratio of about 20 at k = 4), run on FP64 products.
+ *   1D: three FP32 numbers (72 bits), error as with FP64 exponentials; the same fallback.
  * KBL_FP32_MIXED: Maxwellians, envelopes and velocity sums in FP32 (2D: each thread sums its
  *   16 velocity nodes, the threads' sums meet in a pairwise tree, at most 25 roundings of the sum
  *   of magnitudes, which for these single-signed sums is the sum itself: <= 1.5e-6 relative;

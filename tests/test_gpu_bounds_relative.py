@@ -144,3 +144,32 @@ def test_line_states_equal_to_rounding(nu, k):
             ref = (q * f).sum() * h
             err[b, e] = float((L(got[b, 0, e]) - ref) / ref)
     assert abs(err[1].mean() - err[0].mean()) < 2.0 ** -53, err.mean(1)
+
+
+def _rms_sets():
+    rng = np.random.default_rng(21)
+    E, n = 24, 33
+    u = lambda a, b, s=(E, n): rng.uniform(a, b, s)
+    x, y = u(-1, 1), u(-1, 1)
+    g = u(-0.1, 0.1, (8, E, 1))
+    smooth = _cons(1 + g[0] * x + g[1] * y, 0.3 + g[2] * x + g[3] * y, -0.2 + g[4] * x + g[5] * y, 1 + g[6] * x + g[7] * y)
+    r, t = u(0.5, 1.5, (E, 1)), u(0.5, 1.5, (E, 1))
+    nodes = _cons(r * u(0.8, 1.2), u(-1, 1, (E, 1)) + u(-0.2, 0.2), u(-1, 1, (E, 1)) + u(-0.2, 0.2), t * u(0.8, 1.2))
+    factors = _cons(u(0.1, 2.0), u(-1, 1), u(-1, 1), u(0.5, 2.0))
+    return {"smooth": (smooth, 3e-16), "nodes": (nodes, 3e-16), "factors": (factors, 4.5e-16)}
+
+
+@pytest.mark.parametrize("nu,k,quad", [(32, 4.0, 0), (33, 4.0, 1), (40, 4.0, 0), (48, 4.0, 0), (64, 8.0, 0)])
+@pytest.mark.parametrize("which", ["smooth", "nodes", "factors"])
+def test_stated_errors(which, nu, k, quad):
+    """The rms errors that include/kbl.h states for the pairs: below 3e-16 for smooth and moderately
+    scattered states over all bounds and over the lower ones of density and energy; below 4.5e-16 where
+    the states of a stencil differ by factors."""
+    S, stated = _rms_sets()[which]
+    got = _bounds(S, nu, k, quad)
+    err = np.zeros(got.shape)
+    for e in range(len(S)):
+        ref, mag, _, _, _ = _reference(S[e], nu, k, quad)
+        err[:, :, e] = (np.abs(got[:, :, e].astype(L) - ref) / mag).astype(float)
+    rms, low = np.sqrt((err ** 2).mean()), np.sqrt((err[0, [0, 3]] ** 2).mean())
+    assert rms < stated and low < stated, (rms, low)
