@@ -543,7 +543,7 @@ def run_batched(args, rank, world, steps=None, warmup=None):
                     "d2h_bytes_per_step": w0.nbytes,
                     "call": "kbl_batch_run_host, 1 step, pinned host buffers, copies overlapped by problem groups"},
             "gpu_launches": launches,
-            "form": {"timed": "one persistent launch per phase, 14 per step, in one graph",
+            "form": {"timed": "one persistent launch per phase, 13 per step, in one graph",
                      "one_launch_ms_per_step": one_launch_ms,
                      "one_launch": "the whole step as one persistent launch with per-problem dataflow"},
             "roofline": {"bound": "alu", "achieved": round(achieved, 3), "peak": round(peak, 3),

@@ -232,9 +232,9 @@ cudaError_t dalloc(T** p, size_t count)
 // kernel joins them.  Traces and bounds are programmatic dependents on the main branch: a bounds
 // block is resident when the stage before it ends.  The stage kernel is an ordinary launch behind
 // both.  Step time against one main chain traces -> residual -> bounds -> stage of programmatic
-// dependents: 200 1D P3 elements in FP64 82 us there, 62 here; 16^2 P3 mixed 51 and 45, 32^2 FP64
-// 274 and 243; at 128^2 the bounds fill the chip and little is left to hide: mixed 515 and 513,
-// FP64 3025 and 3001 (so no rule on the size).  FP32 bounds on more than 32 velocity nodes per axis
+// dependents, steps back to back: 200 1D P3 elements in FP64 85 us there, 68 here; 16^2 P3 mixed 64 and
+// 55, 32^2 FP64 260 and 250; at 128^2 the bounds fill the chip and little is left to hide: mixed 509 and
+// 507, FP64 2920 and 2897 (so no rule on the size).  FP32 bounds on more than 32 velocity nodes per axis
 // keep the one chain (ctx->pdl_chain: residuals and stages programmatic dependents as well): their
 // blocks of 256 threads wait for room beside the residual's, and a branch cost more than it hid (200^2
 // P3, 48 nodes: 5.66 ms per step in the chain, 5.83 with the branch).

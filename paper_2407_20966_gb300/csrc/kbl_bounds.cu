@@ -89,7 +89,7 @@ k_bounds2d_f32(const double* __restrict__ w, const double* __restrict__ wf, Mesh
 // ---------------------------------------------------------------------------
 // 1D, FP64: one block per element, the velocity nodes over its threads (kbl_bounds64_body.cuh).  Bound by
 // instruction issue; an FP64 exponential and quotient per (state, node) held the FP64 pipe 42 slots
-// each: 374 -> 75 us per launch at 300 P4 elements, 2048 nodes, 23 -> 12 us at 200 P3, 64 nodes.
+// each: 374 -> 74 us per launch at 300 P4 elements, 2048 nodes, 23 -> 12 us at 200 P3, 64 nodes.
 // ---------------------------------------------------------------------------
 template <int N, int NT, bool WIDE = false>
 __global__ void __launch_bounds__(NT)

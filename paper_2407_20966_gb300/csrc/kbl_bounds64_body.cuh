@@ -317,7 +317,7 @@ __device__ __forceinline__ void bounds2d_f64_core(Bounds2dF64Smem<NST, NX>& sm, 
 //
 //   row tables   a_i(u) = A_i 2^-t(u), c_i = C_i a_i, b_i(v) = 2^-t(v), t = (u - U)^2 log2(e)/(2 theta),
 //                t in 64-bit fixed point by second differences (exact additions), 2^-t by a table of
-//                64 exact knots and a polynomial on float pairs
+//                128 exact knots and a polynomial on float pairs
 //   pass 1       M = max_i fl(a_hi b_hi) (min alike; c b alike): the FP32 envelope
 //   pass 2       E = max_i [a_hi b_hi - M + a_hi b_lo + a_lo b_hi] by FMAs, the first of which forms
 //                a_hi b_hi - M with one rounding: the envelope is M + E, its winner decided to
@@ -325,7 +325,8 @@ __device__ __forceinline__ void bounds2d_f64_core(Bounds2dF64Smem<NST, NX>& sm, 
 //   moments      the nodes' values in error-free FP32 sums along rows and columns, those in FP64;
 //                the quadrature weights are in the tables already
 //
-// Measured at 128^2 P3, 32^2 grid: 0.85 ms per launch; 0.87 with both axes' grid coefficients in one
+// Measured at 128^2 P3, 32^2 grid: 0.83 ms per launch (0.85 while table entries carried their rounding
+// errors along the row, the base of the figures that follow); 0.87 with both axes' grid coefficients in one
 // thread per state, 0.95 with the y table's values stored twice (a
 // 128-bit shared load takes four wavefronts however many lanes share its addresses, and the passes
 // wait on them: 6.9k of 19k clocks per element), 1.08 with the moments node by node in FP64 and the
@@ -335,7 +336,8 @@ __device__ __forceinline__ void bounds2d_f64_core(Bounds2dF64Smem<NST, NX>& sm, 
 // 0.57 at 24.
 // What bounds it: per (state, node) 14 FP32 products/FMAs (packed two to an instruction, two
 // neighbouring x nodes) and four three-input min/max, 7 + 4 issue slots: about half the launch; the
-// states' FP64 chains, tables and sums the other half.
+// states' FP64 chains, tables and sums the other half.  Counters at 64^2 P3: issue slots 56% busy, FP64
+// pipe 46%, ALU 34%, FMA pipe 30%; 128 registers, four blocks per SM.
 //
 // Elements outside the range of the pairs (a state more than 2^240 below its peak inside the box,
 // constants beyond +-2^60 of the largest, a lower density sum below 2^-40 of the largest state's)
